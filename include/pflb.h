@@ -67,13 +67,14 @@ enum { PFLB_FIELD_PHI = 0, PFLB_FIELD_RHO = 1, PFLB_FIELD_P = 2,
 
 /* Step kernels.  Every kind computes the same step; they differ in how the
  * populations reach the arithmetic:
- *   PFLB_KERNEL_PIPE (default): the fused z-marching pass with each thread's
+ *   PFLB_KERNEL_PIPE (default): two kernels per step, phi of every cell
+ *     and then the update, for any extent and boundaries; lattices whose h
+ *     populations are larger than twice the L2 cache, with periodic x and nx
+ *     a multiple of 4, run one fused z-marching kernel instead, each thread's
  *     populations of the next planes copied into shared memory one plane
  *     ahead (cp.async in 16-byte chunks; 8-byte chunks at FP16/BF16 storage
- *     when nx is not a multiple of 8), 32 x 4 tiles, pair form of the
- *     collision, each block's wall nodes updated after its march (one
- *     launch per step); periodic x and nx a multiple of 4, otherwise
- *     PFLB_KERNEL_FUSED runs;
+ *     when nx is not a multiple of 8), 32 x 4 tiles.  Both use the pair form
+ *     of the collision;
  *   PFLB_KERNEL_FUSED: one fused z-marching pass with direct loads;
  *   PFLB_KERNEL_TWOPASS: a phi pass followed by a per-cell pass;
  *   PFLB_KERNEL_FUSED_TMA: the fused pass with h staged through shared
@@ -230,9 +231,8 @@ pflb_status pflb_set_kernel(pflb_lattice *L, int kind, int bx, int by, int lz);
  * rho_b (Gamma_i(u_b) - w_i), streamed as usual (bounce-back at solid
  * links), and whatever streams into it is discarded.  Boundary cells carry
  * no diagnostics and read back their boundary state.  First-order accurate
- * (equilibrium boundary).  Lattices with open boundaries run the fused or
- * two-pass kernel (not the TMA one); in a batch their boundary states are
- * formed by one extra kernel per step over all such lattices. */
+ * (equilibrium boundary).  Lattices with open boundaries run every
+ * kernel kind but the TMA one. */
 enum { PFLB_XBC_PRESSURE = 1, PFLB_XBC_VELOCITY = 2 };
 typedef struct {
   int type;        /* PFLB_XBC_PRESSURE or PFLB_XBC_VELOCITY */
@@ -371,20 +371,17 @@ pflb_status pflb_fields_noalloc(int nx, int ny, int nz, const float *h_dev, cons
                                 pflb_diag_t *diag_out, void *cuda_stream);
 
 /* ------------------------------------------------------------- batches
- * Many independent lattices (of any sizes) advanced together by persistent
- * kernels: a grid of (SMs x blocks per SM) blocks pulls work items -- one
- * per (lattice, tile column, chunk of z planes) -- from a device work list,
- * so small lattices that could not fill the GPU on their own share it.
- * Lattices that PFLB_KERNEL_PIPE can run (periodic x, nx a multiple of 4)
- * are marched by its pipelined per-cell code, 32 x 4
- * tiles with an automatic number of planes, their wall nodes by a second
- * small kernel; the others by the fused tile march with the launch shape
- * below.  No work item reads another lattice, so a lattice's result does
- * not depend on what it is batched with: it is bit-identical to the same
- * lattice in a batch of its own.  Against pflb_step on that lattice it
- * agrees to rounding (the two kernels are compiled separately and may
- * contract different multiply-adds).  Plain steps are replayed from a
- * captured CUDA graph of 16 steps.  The batch does not own the lattices;
+ * Many independent lattices (of any sizes) advanced together.  Lattices of
+ * less than 400000 cells are put into groups of up to 600000 cells, each
+ * stepped by the two kernels of the default kind over one work list, one item
+ * per block (a range of one lattice's cells, wall nodes or boundary cells), so
+ * that small lattices that could not fill the GPU on their own share it and a
+ * group's state stays in L2 from step to step.  Larger lattices are stepped
+ * one after the other by their own kernels.  No work item reads another
+ * lattice, so a lattice's result does not depend on what it is batched with:
+ * it is bit-identical to the same lattice in a batch of its own.  Against
+ * pflb_step on that lattice it agrees to rounding (the kernels are compiled
+ * separately and may contract different multiply-adds).  The batch does not own the lattices;
  * they must outlive it, share one storage type, and appear once.  Work is
  * ordered on the batch stream (cuda_stream, or a stream the batch creates
  * when NULL), after and before the lattices' own streams. */
@@ -393,10 +390,11 @@ typedef struct pflb_batch pflb_batch;
 pflb_status pflb_batch_create(pflb_lattice *const *lattices, int count, void *cuda_stream,
                               pflb_batch **out);
 
-/* Launch shape of the fused tile march: bx * by threads per block (same
- * rules as pflb_set_kernel), lz planes per work item, blocks per SM (0 = as
- * many as fit, at most 4); zeros keep the current values (default
- * 32 x 4 x 16, 0). */
+/* Launch shape of the groups: a work item of bulk cells holds bx * by * lz / 8
+ * of them (bx and by under the rules of pflb_set_kernel); zeros keep the
+ * current values (default 32 x 4 x 16).  blocks_per_sm is accepted (>= 0) and
+ * bounds the value that pflb_batch_tune reports; the grids hold one block per
+ * item. */
 pflb_status pflb_batch_set_launch(pflb_batch *b, int bx, int by, int lz, int blocks_per_sm);
 
 /* Autotuner: times trial_steps steps of each of a fixed set of launch shapes

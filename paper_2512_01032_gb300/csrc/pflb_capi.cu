@@ -30,20 +30,16 @@ struct pflb_batch {
   std::vector<Lattice *> lats;
   int storage = PFLB_STORAGE_FP32;
   pflb::BatchDev dev;
-  size_t desc_bytes = 0;
-  size_t items_cap = 0;
-  int blocks_per_sm = 0;  // requested; 0 = as many as fit, at most 4
-  int per_sm = 0;         // in use (the grid may be smaller when items are few)
-  int nsm = 0;
+  std::vector<pflb::BatchGroup> groups;  // small lattices, stepped together
+  std::vector<int> alone;                // lattices that fill the GPU by themselves
+  std::vector<char> open;                // open boundaries the work lists were built for
+  size_t desc_bytes = 0, items_cap = 0;
+  int blocks_per_sm = 0;  // requested; 0 = as many as fit
+  int per_sm = 0;
   bool own_stream = false;
   cudaEvent_t ev = nullptr;
-  cudaGraphExec_t graph = nullptr;  // kGraphSteps plain steps
-  int graph_nxbc = -1;               // open-boundary lattice count the graph was captured for
-  int graph_pmask = -1;              // A-A parities of the pipelined lattices at capture
-  std::vector<char> pipe_set;        // lattices the work lists were built to march pipelined
   bool poisoned = false;
 };
-static constexpr int kGraphSteps = 16;
 
 namespace {
 
@@ -124,6 +120,23 @@ size_t storage_bytes(int storage) {
 size_t compute_bytes(int storage) { return storage == PFLB_STORAGE_FP64 ? 8 : 4; }
 // h slots per cell: the 16-bit formats keep the rest population's remainder.
 size_t h_slots_of(int storage) { return storage_bytes(storage) == 2 ? 20 : 19; }
+
+// Whether the default kind takes the two-phase step where the pipelined march
+// could run too: up to twice the L2 cache of h populations.  Measured (us per
+// step, march / two phases): FP32 drop 64^3 24.7 / 14.4, channel 384 x 80 x 80
+// (187 MB of h) 201 / 172, drop 144^3 (227 MB) 203 / 201; beyond, drop
+// 160^3 (311 MB) 253 / 286, channel 512 x 128 x 128 (638 MB) 554 / 574; BF16
+// drop 128^3 (84 MB) 126 / 119, drop 176^3 (218 MB) 319 / 312, drop 192^3
+// (283 MB) 367 / 395.
+bool h_stays_in_l2(const Lattice *L) {
+  int dev = 0, l2 = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return (double)h_slots_of(L->p.storage) * L->N * L->elem <= 2.0 * l2;
+}
 
 // Planes per block in effect: the requested value, else the automatic one.
 int resolve_lz(Lattice *L) {
@@ -622,6 +635,7 @@ pflb_status pflb_create(const pflb_geometry *geom, const pflb_params *params, vo
     return fail(PFLB_ERR_CUDA, std::string("upload failed: ") + cudaGetErrorString(e));
   }
   make_tmaps(L);
+  L->h_in_l2 = h_stays_in_l2(L);
   L->lz = resolve_lz(L);
   L->wcell_h.swap(hg.wcell);
   e = ensure_wall_lists(L, L->aux);  // nothing on the lattice's stream reads them yet
@@ -850,9 +864,9 @@ pflb_status pflb_get_kernel(const pflb_lattice *L, int out[4]) {
   if (!out) return fail(PFLB_ERR_ARG, "null output");
   const bool tma = L->kernel == PFLB_KERNEL_FUSED_TMA && L->p.storage == PFLB_STORAGE_FP32 &&
                    L->tma_ok && !L->bc_on;
-  const bool pipe = pflb::pipe_kernel_runs(*L);
-  // the kind that runs: the pipelined and TMA kernels fall back to the
-  // fused one where they do not apply
+  const bool pipe = L->kernel == PFLB_KERNEL_PIPE;
+  // the kind that runs: the TMA kernel falls back to the fused one where it
+  // does not apply
   out[0] = pipe || tma || L->kernel == PFLB_KERNEL_TWOPASS ? L->kernel : PFLB_KERNEL_FUSED;
   out[1] = tma ? 32 : (pipe ? 32 : L->bx);
   out[2] = tma ? 8 : (pipe ? 4 : L->by);
@@ -1140,123 +1154,84 @@ static pflb_status batch_fail(pflb_batch *b, cudaError_t e, const char *what) {
     if (e_ != cudaSuccess) return batch_fail(b, e_, #call);  \
   } while (0)
 
-static void batch_drop_graph(pflb_batch *b) {
-  if (b->graph) cudaGraphExecDestroy(b->graph);
-  b->graph = nullptr;
-}
+// A lattice of this many cells or more fills the GPU by itself: it is
+// stepped by its own kernels, all steps of a call in a row.
+static constexpr long long kAloneCells = 400000;
+// Cells of a group of smaller ones: enough to fill the GPU, few enough that
+// their state stays in L2 from step to step.
+static constexpr long long kGroupCells = 600000;
 
-// Which lattices of the batch the pipelined march can run (the others use
-// the fused tile march of k_batch).
-static std::vector<char> batch_pipe_set(const pflb_batch *b) {
+static std::vector<char> batch_open_set(const pflb_batch *b) {
   std::vector<char> on(b->lats.size());
-  for (size_t l = 0; l < b->lats.size(); ++l) on[l] = pflb::pipe_layout_ok(*b->lats[l]) ? 1 : 0;
+  for (size_t l = 0; l < b->lats.size(); ++l) on[l] = b->lats[l]->bc_on ? 1 : 0;
   return on;
 }
 
-// Work lists of the pipelined lattices (tile columns of 32 x 4 in chunks of
-// plz planes, plz minimising rounds of resident blocks x (plz + 0.6) as for
-// a single lattice; wall nodes in chunks of 128), and their grid.
-static pflb_status batch_build_pipe_items(pflb_batch *b) {
+// Groups, their work lists and the upload of these.  Open and periodic
+// lattices are in different groups (they run different compiled variants),
+// so what a lattice runs does not depend on what it is batched with.
+static pflb_status batch_build_items(pflb_batch *b) {
   BCK(b, cudaStreamSynchronize(b->dev.stream));  // the old lists may still be in use
-  std::vector<int4> items;
-  std::vector<int2> witems;
-  long long cols = 0;
-  int maxz = 1;
-  for (int l = 0; l < (int)b->lats.size(); ++l) {
-    if (!b->pipe_set[l]) continue;
-    const Lattice *L = b->lats[l];
-    cols += (long long)((L->nx + 31) / 32) * ((L->ny + 3) / 4);
-    maxz = std::max(maxz, L->nz);
-    for (int r = 0; r < L->nw; r += 128) witems.push_back(make_int2(l, r));
-  }
-  const int per = dispatch_storage(b->storage, [&](auto *s_, auto *r_) {
-    PFLB_SR_TYPES
-    return pflb::batch_pipe_blocks_per_sm<S, R>();
-  });
-  const long long slots = (long long)per * b->nsm;
-  int best = 8;
-  double best_cost = 1e300;
-  for (int lz = std::min(32, maxz); lz >= 2 && cols > 0; --lz) {
-    long long blocks = 0;
-    for (int l = 0; l < (int)b->lats.size(); ++l)
-      if (b->pipe_set[l]) {
-        const Lattice *L = b->lats[l];
-        blocks += (long long)((L->nx + 31) / 32) * ((L->ny + 3) / 4) * ((L->nz + lz - 1) / lz);
+  b->groups.clear();
+  b->alone.clear();
+  b->open = batch_open_set(b);
+  for (int want = 0; want < 2; ++want) {
+    long long cells = kGroupCells;
+    for (int l = 0; l < (int)b->lats.size(); ++l) {
+      const Lattice *L = b->lats[l];
+      if ((int)L->bc_on != want) continue;
+      if (L->N >= kAloneCells) {
+        b->alone.push_back(l);
+        continue;
       }
-    const double cost = (double)((blocks + slots - 1) / slots) * (lz + 0.6);
-    if (cost < best_cost - 1e-9) {
-      best_cost = cost;
-      best = lz;
+      if (cells + L->N > kGroupCells) {
+        b->groups.emplace_back();
+        b->groups.back().open = want != 0;
+        cells = 0;
+      }
+      b->groups.back().lats.push_back(l);
+      cells += L->N;
     }
   }
-  b->dev.plz = best;
-  std::vector<int4> items8;  // lattices staged in 8-byte chunks
-  for (int l = 0; l < (int)b->lats.size(); ++l) {
-    if (!b->pipe_set[l]) continue;
-    const Lattice *L = b->lats[l];
-    std::vector<int4> &dst = pflb::pipe_chunk_bytes(*L) == 8 ? items8 : items;
-    for (int z0 = 0; z0 < L->nz; z0 += best)
-      for (int y0 = 0; y0 < L->ny; y0 += 4)
-        for (int x0 = 0; x0 < L->nx; x0 += 32) dst.push_back(make_int4(l, x0, y0, z0));
-  }
-  if (b->dev.pitems) cudaFree(b->dev.pitems);
-  if (b->dev.pitems8) cudaFree(b->dev.pitems8);
-  if (b->dev.witems) cudaFree(b->dev.witems);
-  b->dev.pitems = b->dev.pitems8 = b->dev.witems = nullptr;
-  b->dev.npitems = (int)items.size();
-  b->dev.npitems8 = (int)items8.size();
-  b->dev.nwitems = (int)witems.size();
-  if (!items.empty()) {
-    BCK(b, cudaMalloc(&b->dev.pitems, items.size() * sizeof(int4)));
-    BCK(b, cudaMemcpyAsync(b->dev.pitems, items.data(), items.size() * sizeof(int4),
-                           cudaMemcpyHostToDevice, b->dev.stream));
-  }
-  if (!items8.empty()) {
-    BCK(b, cudaMalloc(&b->dev.pitems8, items8.size() * sizeof(int4)));
-    BCK(b, cudaMemcpyAsync(b->dev.pitems8, items8.data(), items8.size() * sizeof(int4),
-                           cudaMemcpyHostToDevice, b->dev.stream));
-  }
-  if (!witems.empty()) {
-    BCK(b, cudaMalloc(&b->dev.witems, witems.size() * sizeof(int2)));
-    BCK(b, cudaMemcpyAsync(b->dev.witems, witems.data(), witems.size() * sizeof(int2),
-                           cudaMemcpyHostToDevice, b->dev.stream));
-  }
-  b->dev.pgrid = (int)std::max(
-      1LL, std::min<long long>(std::max(b->dev.npitems, b->dev.npitems8), slots));
-  return PFLB_OK;
-}
-
-// Work list for the current launch shape, and the persistent grid size.
-static pflb_status batch_build_items(pflb_batch *b) {
-  b->pipe_set = batch_pipe_set(b);
-  pflb_status pst = batch_build_pipe_items(b);
-  if (pst != PFLB_OK) return pst;
+  // cells per bulk item: the launch shape's tile times its planes over 8
+  const int chunk = std::max(64, b->dev.bx * b->dev.by * b->dev.lz / 8 / 64 * 64);
   std::vector<int4> items;
-  const int bx = b->dev.bx, by = b->dev.by, lz = b->dev.lz;
-  for (int l = 0; l < (int)b->lats.size(); ++l) {
-    if (b->pipe_set[l]) continue;
-    const Lattice *L = b->lats[l];
-    for (int z0 = 0; z0 < L->nz; z0 += lz)
-      for (int y0 = 0; y0 < L->ny; y0 += by)
-        for (int x0 = 0; x0 < L->nx; x0 += bx) items.push_back(make_int4(l, x0, y0, z0));
+  for (pflb::BatchGroup &g : b->groups) {
+    auto add = [&](int l, int kind, int count, int per) {
+      for (int o = 0; o < count; o += per)
+        items.push_back(make_int4(l, kind, o, std::min(per, count - o)));
+    };
+    g.first1 = (int)items.size();
+    for (int l : g.lats) {
+      const Lattice *L = b->lats[l];
+      if (L->bc_on) add(l, 1, 2 * L->ny * L->nz, 128);
+    }
+    for (int l : g.lats) add(l, 0, (int)b->lats[l]->N, 1024);
+    g.n1 = (int)items.size() - g.first1;
+    g.first2 = (int)items.size();
+    for (int l : g.lats) add(l, 3, b->lats[l]->nw, 64);
+    for (int l : g.lats) {
+      const Lattice *L = b->lats[l];
+      if (L->bc_on) add(l, 4, 2 * L->ny * L->nz, 64);
+    }
+    for (int l : g.lats) add(l, 2, (int)b->lats[l]->N, chunk);
+    g.n2 = (int)items.size() - g.first2;
   }
   if (items.size() > b->items_cap) {
     if (b->dev.items) cudaFree(b->dev.items);
     b->dev.items = nullptr;
+    b->items_cap = 0;
     BCK(b, cudaMalloc(&b->dev.items, items.size() * sizeof(int4)));
     b->items_cap = items.size();
   }
-  b->dev.nitems = (int)items.size();
   if (!items.empty())
     BCK(b, cudaMemcpyAsync(b->dev.items, items.data(), items.size() * sizeof(int4),
                            cudaMemcpyHostToDevice, b->dev.stream));
   const int fit = dispatch_storage(b->storage, [&](auto *s_, auto *r_) {
     PFLB_SR_TYPES
-    return pflb::batch_max_blocks_per_sm<S, R>(bx, by);
+    return pflb::batch_blocks_per_sm<S, R>();
   });
-  b->per_sm = b->blocks_per_sm > 0 ? std::min(b->blocks_per_sm, fit) : std::min(fit, 4);
-  b->dev.grid = std::max(1, std::min(b->dev.nitems, b->per_sm * b->nsm));
-  batch_drop_graph(b);
+  b->per_sm = b->blocks_per_sm > 0 ? std::min(b->blocks_per_sm, fit) : fit;
   BCK(b, cudaStreamSynchronize(b->dev.stream));
   return PFLB_OK;
 }
@@ -1278,10 +1253,6 @@ extern "C" pflb_status pflb_batch_create(pflb_lattice *const *lattices, int coun
   if (!b) return fail(PFLB_ERR_OOM, "host allocation failed");
   for (int l = 0; l < count; ++l) b->lats.push_back(lattices[l]);
   b->storage = lattices[0]->p.storage;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&b->nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (b->nsm < 1) b->nsm = 1;
   cudaError_t e = cudaSuccess;
   if (cuda_stream) {
     b->dev.stream = (cudaStream_t)cuda_stream;
@@ -1296,11 +1267,8 @@ extern "C" pflb_status pflb_batch_create(pflb_lattice *const *lattices, int coun
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaMalloc(&b->dev.descs, 2 * (size_t)count * b->desc_bytes);
   if (e == cudaSuccess) e = cudaMalloc((void **)&b->dev.par0, count * sizeof(int));
-  if (e == cudaSuccess) e = cudaMalloc((void **)&b->dev.counter, sizeof(int));
-  if (e == cudaSuccess) e = cudaMalloc((void **)&b->dev.pcounter, sizeof(int));
-  if (e == cudaSuccess) e = cudaMalloc((void **)&b->dev.bstep, sizeof(int));
+  if (e == cudaSuccess) e = cudaMalloc((void **)&b->dev.bstep, count * sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc((void **)&b->dev.xspecs, count * sizeof(pflb::XbcSpec));
-  if (e == cudaSuccess) e = cudaMalloc((void **)&b->dev.xlist, count * sizeof(int));
   if (e != cudaSuccess) {
     pflb_batch_destroy(b);
     cudaGetLastError();
@@ -1332,12 +1300,11 @@ extern "C" pflb_status pflb_batch_set_launch(pflb_batch *b, int bx, int by, int 
   return batch_build_items(b);
 }
 
-// Runs nsteps on the batch stream (graph replay for the plain steps).
+// Runs nsteps on the batch stream.
 static pflb_status batch_run(pflb_batch *b, int64_t nsteps, bool diag_last) {
   const int n = (int)b->lats.size();
   // open boundaries switched on or off since the work lists were built
-  // move a lattice between the pipelined and the fused march
-  if (batch_pipe_set(b) != b->pipe_set) {
+  if (batch_open_set(b) != b->open) {
     pflb_status st = batch_build_items(b);
     if (st != PFLB_OK) return st;
   }
@@ -1347,80 +1314,52 @@ static pflb_status batch_run(pflb_batch *b, int64_t nsteps, bool diag_last) {
     BCK(b, cudaEventRecord(b->ev, L->stream));
     BCK(b, cudaStreamWaitEvent(b->dev.stream, b->ev, 0));
   }
-  std::vector<char> host(2 * (size_t)n * b->desc_bytes);
-  std::vector<int> par(n);
-  dispatch_storage(b->storage, [&](auto *s_, auto *r_) {
-    PFLB_SR_TYPES
-    pflb::batch_build_descs<S, R>(b->lats.data(), n, host.data());
-    return 0;
-  });
-  for (int l = 0; l < n; ++l) par[l] = (int)(b->lats[l]->step & 1);
-  // parities the pipelined lattices start this call at (one march launch
-  // per parity present at each step)
-  int pmask = 0;
-  for (int l = 0; l < n; ++l)
-    if (b->pipe_set[l]) pmask |= 1 << par[l];
-  b->dev.pmask = pmask;
-  if (pmask != b->graph_pmask) batch_drop_graph(b);
-  // open x boundaries: specs of every lattice (type 0 = periodic) and the
-  // list of those that have them; the values may change between calls
-  std::vector<pflb::XbcSpec> specs(n);
-  std::vector<int> xlist;
-  for (int l = 0; l < n; ++l) {
-    const Lattice *L = b->lats[l];
-    specs[l] = pflb::xbc_spec(*L, L->step);
-    if (L->bc_on) xlist.push_back(l);
-  }
-  b->dev.nxbc = (int)xlist.size();
-  if (b->dev.nxbc != b->graph_nxbc) batch_drop_graph(b);
-  BCK(b, cudaMemcpyAsync(b->dev.xspecs, specs.data(), n * sizeof(pflb::XbcSpec),
-                         cudaMemcpyHostToDevice, b->dev.stream));
-  if (!xlist.empty())
-    BCK(b, cudaMemcpyAsync(b->dev.xlist, xlist.data(), xlist.size() * sizeof(int),
-                           cudaMemcpyHostToDevice, b->dev.stream));
-  BCK(b, cudaMemcpyAsync(b->dev.descs, host.data(), host.size(), cudaMemcpyHostToDevice,
-                         b->dev.stream));
-  BCK(b, cudaMemcpyAsync(b->dev.par0, par.data(), n * sizeof(int), cudaMemcpyHostToDevice,
-                         b->dev.stream));
-  BCK(b, cudaMemsetAsync(b->dev.bstep, 0, sizeof(int), b->dev.stream));
-  // tpar: parity of the batch step (the device counter bstep starts at 0
-  // with each call and advances by one per step)
-  auto launch = [&](bool diag, int tpar) {
-    return dispatch_storage(b->storage, [&](auto *s_, auto *r_) {
+  if (!b->groups.empty()) {
+    std::vector<char> host(2 * (size_t)n * b->desc_bytes);
+    dispatch_storage(b->storage, [&](auto *s_, auto *r_) {
       PFLB_SR_TYPES
-      return pflb::batch_launch_step<S, R>(b->dev, diag, tpar);
+      pflb::batch_build_descs<S, R>(b->lats.data(), n, host.data());
+      return 0;
     });
-  };
-  int64_t plain = nsteps - (diag_last ? 1 : 0);
-  int64_t t = 0;
-  if (plain >= kGraphSteps && !b->graph) {
-    cudaGraph_t g = nullptr;
-    BCK(b, cudaStreamBeginCapture(b->dev.stream, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = cudaSuccess;
-    for (int k = 0; k < kGraphSteps && e == cudaSuccess; ++k) e = launch(false, k & 1);
-    cudaError_t e2 = cudaStreamEndCapture(b->dev.stream, &g);
-    if (e == cudaSuccess) e = e2;
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&b->graph, g, 0);
-    if (g) cudaGraphDestroy(g);
-    if (e != cudaSuccess) return batch_fail(b, e, "graph capture");
-    b->graph_nxbc = b->dev.nxbc;
-    b->graph_pmask = b->dev.pmask;
-  }
-  // replays come first, so each starts at an even batch step (kGraphSteps
-  // is even), as the captured parities assume
-  while (plain >= kGraphSteps) {
-    BCK(b, cudaGraphLaunch(b->graph, b->dev.stream));
-    plain -= kGraphSteps;
-    t += kGraphSteps;
-  }
-  for (; plain > 0; --plain, ++t) BCK(b, launch(false, (int)(t & 1)));
-  if (diag_last) BCK(b, launch(true, (int)(t & 1)));
-  for (Lattice *L : b->lats) {
-    L->step += nsteps;
-    if (diag_last) {
-      L->last_diag_step = L->step - 1;
-      L->ndiag++;
+    std::vector<int> par(n);
+    std::vector<pflb::XbcSpec> specs(n);
+    for (int l = 0; l < n; ++l) {
+      par[l] = (int)(b->lats[l]->step & 1);
+      specs[l] = pflb::xbc_spec(*b->lats[l], b->lats[l]->step);
     }
+    BCK(b, cudaMemcpyAsync(b->dev.xspecs, specs.data(), n * sizeof(pflb::XbcSpec),
+                           cudaMemcpyHostToDevice, b->dev.stream));
+    BCK(b, cudaMemcpyAsync(b->dev.descs, host.data(), host.size(), cudaMemcpyHostToDevice,
+                           b->dev.stream));
+    BCK(b, cudaMemcpyAsync(b->dev.par0, par.data(), n * sizeof(int), cudaMemcpyHostToDevice,
+                           b->dev.stream));
+    BCK(b, cudaMemsetAsync(b->dev.bstep, 0, n * sizeof(int), b->dev.stream));
+    for (size_t gi = 0; gi < b->groups.size(); ++gi)
+      for (int64_t t = 0; t < nsteps; ++t)
+        BCK(b, dispatch_storage(b->storage, [&](auto *s_, auto *r_) {
+          PFLB_SR_TYPES
+          return pflb::batch_launch_step<S, R>(b->dev, b->groups[gi], (int)gi,
+                                               diag_last && t == nsteps - 1, (int)(t & 1));
+        }));
+    for (const pflb::BatchGroup &g : b->groups)
+      for (int l : g.lats) {
+        Lattice *L = b->lats[l];
+        L->step += nsteps;
+        if (diag_last) {
+          L->last_diag_step = L->step - 1;
+          L->ndiag++;
+        }
+      }
+  }
+  for (int l : b->alone) {
+    Lattice *L = b->lats[l];
+    const cudaStream_t own = L->stream;
+    L->stream = b->dev.stream;
+    cudaError_t e = cudaSuccess;
+    for (int64_t t = 0; t < nsteps && e == cudaSuccess; ++t)
+      e = do_step(L, diag_last && t == nsteps - 1);
+    L->stream = own;
+    BCK(b, e);
   }
   // later work on each lattice's own stream comes after the batch
   BCK(b, cudaEventRecord(b->ev, b->dev.stream));
@@ -1476,10 +1415,7 @@ extern "C" pflb_status pflb_batch_tune(pflb_batch *b, int trial_steps, int best[
 extern "C" void pflb_batch_destroy(pflb_batch *b) {
   if (!b) return;
   if (b->dev.stream) cudaStreamSynchronize(b->dev.stream);
-  batch_drop_graph(b);
-  void *ptrs[] = {b->dev.descs,   b->dev.par0,   b->dev.items,  b->dev.counter,
-                  b->dev.bstep,   b->dev.xspecs, b->dev.xlist,  b->dev.pitems,
-                  b->dev.pitems8, b->dev.witems, b->dev.pcounter};
+  void *ptrs[] = {b->dev.descs, b->dev.par0, b->dev.items, b->dev.bstep, b->dev.xspecs};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   if (b->ev) cudaEventDestroy(b->ev);

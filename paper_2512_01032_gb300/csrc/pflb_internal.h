@@ -48,6 +48,7 @@ struct Lattice {
   int64_t last_diag_step = -1;
   int diag_every = 0;         // pflb_step accumulates diagnostics every k-th step
   int kernel = PFLB_KERNEL_PIPE;
+  bool h_in_l2 = false;       // h is small enough to stay in L2 (phase_kernel_runs)
   int bx = 32, by = 4, lz = 16;   // lz: planes per block in effect
   int lz_req = 0;                  // requested planes per block, 0 = automatic
   // open x boundaries (reading R22)
@@ -79,30 +80,22 @@ struct XbcSpec {
   long long step0;    // step of the launch (batches add the batch step)
 };
 
+// Lattices of a batch stepped by the same launches: a range of phase-1 items
+// and one of phase-2 items (int4: lattice, kind, first, count).
+struct BatchGroup {
+  int first1 = 0, n1 = 0, first2 = 0, n2 = 0;
+  bool open = false;  // open x boundaries (all of the group or none)
+  std::vector<int> lats;
+};
+
 struct BatchDev {
   void *descs = nullptr;   // [nlat][2] step descriptors (Args), both parities
   int *par0 = nullptr;     // [nlat] parity of each lattice at batch step 0
-  void *items = nullptr;   // [nitems] int4 (lattice, x0, y0, z0)
-  int nitems = 0;
-  int *counter = nullptr;  // work-list cursor, reset before each step
-  int *bstep = nullptr;    // batch steps since par0 was set
-  int bx = 32, by = 4, lz = 16, grid = 0;
-  cudaStream_t stream = nullptr;
+  void *items = nullptr;   // the work lists of all groups
+  int *bstep = nullptr;    // [nlat] batch steps of each group since the call began
   XbcSpec *xspecs = nullptr;  // [nlat] open-boundary specs (type 0: periodic x)
-  int *xlist = nullptr;       // [nxbc] lattices with open boundaries
-  int nxbc = 0;
-  // lattices run by the pipelined march (pipe_layout_ok): their own work
-  // list of 32 x 4 tile columns in chunks of plz planes, and their wall
-  // nodes in chunks of 128 records (int2: lattice, first record)
-  void *pitems = nullptr;
-  int npitems = 0;
-  void *pitems8 = nullptr;  // the same for lattices staged in 8-byte chunks
-  int npitems8 = 0;
-  int *pcounter = nullptr;
-  int plz = 8, pgrid = 0;
-  int pmask = 0;  // bit q: a pipelined lattice starts the batch call at A-A parity q
-  void *witems = nullptr;
-  int nwitems = 0;
+  int bx = 32, by = 4, lz = 16;
+  cudaStream_t stream = nullptr;
 };
 
 // The pipelined step kernel runs with periodic x and nx a multiple of 4 (its
@@ -114,8 +107,14 @@ inline bool pipe_layout_ok(const Lattice &L) { return !L.bc_on && L.nx % 4 == 0;
 inline int pipe_chunk_bytes(const Lattice &L) {
   return (L.elem == 2 && L.nx % 8 != 0) ? 8 : 16;
 }
+// The default kind runs the pipelined march on lattices whose h populations
+// do not stay in L2 between two kernels, where its layout allows it, and the
+// two-phase step on all others.
 inline bool pipe_kernel_runs(const Lattice &L) {
-  return L.kernel == PFLB_KERNEL_PIPE && pipe_layout_ok(L);
+  return L.kernel == PFLB_KERNEL_PIPE && pipe_layout_ok(L) && !L.h_in_l2;
+}
+inline bool phase_kernel_runs(const Lattice &L) {
+  return L.kernel == PFLB_KERNEL_PIPE && !pipe_kernel_runs(L);
 }
 
 // Sets the thread-local message returned by pflb_last_error().
@@ -155,14 +154,13 @@ template <class S, class R> int max_block_threads();
 template <class S, class R> int auto_lz(const Lattice &L);
 template <class S, class R> cudaError_t mark_xbc(Lattice &L, bool on);
 // Batch: size of one descriptor, host-side descriptor build (2 per lattice,
-// diagnostics pointers for the next diagnostic launch), one step launch,
-// and the occupancy-limited blocks per SM of the batch kernel.
+// diagnostics pointers for the next diagnostic launch), one step of one
+// group, and the resident blocks per SM of its phase-2 kernel.
 template <class S, class R> size_t batch_desc_bytes();
 template <class S, class R> void batch_build_descs(Lattice *const *lats, int n, char *host);
-template <class S, class R> cudaError_t batch_launch_step(const BatchDev &b, bool diag,
-                                                         int tpar);
-template <class S, class R> int batch_max_blocks_per_sm(int bx, int by);
-template <class S, class R> int batch_pipe_blocks_per_sm();
+template <class S, class R> cudaError_t batch_launch_step(const BatchDev &b, const BatchGroup &g,
+                                                         int gi, bool diag, int tpar);
+template <class S, class R> int batch_blocks_per_sm();
 
 }  // namespace pflb
 

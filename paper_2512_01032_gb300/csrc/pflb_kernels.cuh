@@ -44,11 +44,27 @@ enum { COLL_PLAIN = 0, COLL_PAIRS = 1, COLL_X2 = 2, COLL_X2_NOF = 3 };
 #define PFLB_FUSED_MAXNREG 96
 #endif
 
+// Division by a constant known at launch, exact for 0 <= n < 2^31
+// (multiply-high by a 33-bit reciprocal, Granlund and Montgomery 1994).
+struct FastDiv {
+  uint32_t mul, shift;
+};
+inline FastDiv fast_div(uint32_t d) {
+  FastDiv f{0, 0};
+  while ((1ull << f.shift) < d) ++f.shift;
+  f.mul = (uint32_t)(((1ull << 32) * ((1ull << f.shift) - d)) / d + 1);
+  return f;
+}
+__device__ __forceinline__ int div_by(int n, const FastDiv &f) {
+  return (int)((__umulhi((uint32_t)n, f.mul) + (uint32_t)n) >> f.shift);
+}
+
 template <class S, class R>
 struct Args {
   int nx, ny, nz, lz;
   int N;
   int nw;
+  FastDiv dx, dxy;       // by nx and by nx ny
   const S *hin[Q + 1];   // direction bases of the h buffer being read (+ rest remainder)
   S *hout[Q + 1];        // direction bases of the h buffer being written
   S *g[Q];           // direction bases of the g buffer (in place)
@@ -194,8 +210,10 @@ __device__ __forceinline__ void boundary_cell(const Args<S, R> &a, int x, int y,
 // Rest of the update (or macro evaluation) of one fluid cell c at (x, y, z)
 // once its populations are gathered: h[] and g[] hold the streamed
 // populations, phi = sum h, val[1..18] the phi of the 18 neighbours
-// (anything for solid ones), lm/rec the wall data (0 for bulk cells).
-template <class S, class R, bool ODD, int MODE, bool DIAG, bool XBC = false, int PAIRS = COLL_PLAIN>
+// (anything for solid ones; with HAVE, their ghosts), lm/rec the wall data (0
+// for bulk cells).
+template <class S, class R, bool ODD, int MODE, bool DIAG, bool XBC = false, int PAIRS = COLL_PLAIN,
+          bool HAVE = false>
 __device__ __forceinline__ void finish_cell(const Args<S, R> &a, int x, int y, int z, int c,
                                             uint8_t f, uint32_t lm, int rec, const Nbr &nb,
                                             R h[Q], R g[Q], R phi, R val[Q], DiagAcc<R> &acc) {
@@ -220,9 +238,11 @@ __device__ __forceinline__ void finish_cell(const Args<S, R> &a, int x, int y, i
     // sub-voxel walls: links into cut cells and the sample direction c_n
     const uint32_t cw = a.wcut ? a.wcut[rec] : 0u;
     const uint32_t lc = cw & 0x7fffeu;
+    if (!HAVE) {
 #pragma unroll
-    for (int i = 1; i < Q; ++i)
-      if ((lm >> i) & 1u) val[i] = a.ghost[(i - 1) * nw + rec];
+      for (int i = 1; i < Q; ++i)
+        if ((lm >> i) & 1u) val[i] = a.ghost[(i - 1) * nw + rec];
+    }
     // phi_smpl: the node's phi, or for a cut node the average over the
     // parallelepiped on the wall, (1 - s_x) phi + s_x phi(x + c_n)
     R smpl = phi;

@@ -5,9 +5,9 @@
 #include <type_traits>
 
 #include "pflb_async.cuh"
-#include "pflb_batch.cuh"
 #include "pflb_internal.h"
 #include "pflb_kernels.cuh"
+#include "pflb_phase.cuh"
 #include "pflb_pipe.cuh"
 
 namespace pflb {
@@ -48,12 +48,14 @@ static Model<R> make_model(const pflb_params &p) {
 }
 
 template <class S, class R>
-static Args<S, R> make_args(Lattice &L) {
+static Args<S, R> make_args(const Lattice &L, int parity) {
   Args<S, R> a;
   a.nx = L.nx; a.ny = L.ny; a.nz = L.nz; a.lz = L.lz;
   a.N = (int)L.N;
   a.nw = L.nw;
-  const int rd = (int)(L.step & 1);
+  a.dx = fast_div((uint32_t)L.nx);
+  a.dxy = fast_div((uint32_t)L.nx * (uint32_t)L.ny);
+  const int rd = parity;
   for (int i = 0; i < Q + 1; ++i) {
     const bool have = i < h_slots<S>();
     a.hin[i] = have ? (const S *)L.h[rd] + (size_t)i * L.N : nullptr;
@@ -82,6 +84,10 @@ static Args<S, R> make_args(Lattice &L) {
   a.wl = nullptr;  // set by the pipelined launch when its lists are current
   a.wl_start = nullptr;
   return a;
+}
+template <class S, class R>
+static Args<S, R> make_args(const Lattice &L) {
+  return make_args<S, R>(L, (int)(L.step & 1));
 }
 
 // Boundary states of the open x planes for the state the next launch reads.
@@ -180,15 +186,10 @@ static cudaError_t launch_pipe_f(Lattice &L, Args<S, R> &a) {
   if (e != cudaSuccess) return e;
   const dim3 grid((L.nx + PP_BX - 1) / PP_BX, (L.ny + PP_BY - 1) / PP_BY,
                   (L.nz + L.lz - 1) / L.lz);
-  // wall nodes inside the march when the per-block lists match the launch
-  // shape, else by k_wall after it
-  const bool inblock = L.nw > 0 && L.wl && L.wl_lz == L.lz;
-  a.wl = inblock ? L.wl : nullptr;
-  a.wl_start = inblock ? L.wl_start : nullptr;
+  // the wall nodes of each block, listed for the planes per block in effect
+  a.wl = L.nw > 0 ? L.wl : nullptr;
+  a.wl_start = L.nw > 0 ? L.wl_start : nullptr;
   k_pipe<S, R, ODD, DIAG, FORCE, CB><<<grid, PP_NT, sizeof(PipeSmem<S, R, CB>), L.stream>>>(a);
-  e = cudaGetLastError();
-  if (e != cudaSuccess || L.nw == 0 || inblock) return e;
-  k_wall<S, R, ODD, DIAG><<<(L.nw + 127) / 128, 128, 0, L.stream>>>(a);
   return cudaGetLastError();
 }
 
@@ -206,8 +207,79 @@ static cudaError_t launch_pipe_t(Lattice &L, Args<S, R> &a) {
   return launch_pipe_f<S, R, ODD, DIAG, true>(L, a);
 }
 
+// Launch that may be set up while the kernel before it on the stream still
+// runs (the kernel itself waits for that one's end).
+template <class... P, class... A>
+static cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigned block,
+                                    size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// Resident blocks of a kernel on the current device.
+template <class K>
+static cudaError_t resident_blocks(K kernel, int threads, size_t smem, int *blocks) {
+  int dev = 0, sm = 0, per = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem);
+  *blocks = sm * (per > 0 ? per : 1);
+  return e;
+}
+
+// The two-phase step of one lattice.
+template <class S, class R, bool ODD, bool DIAG, bool XBC, bool FORCE>
+static cudaError_t launch_phases_f(Lattice &L, const Args<S, R> &a) {
+  const long long V = phase1_vec<S>(L.N) ? 16 / (int)sizeof(S) : 1;
+  const int plane2 = 2 * L.ny * L.nz;
+  const int nstate = XBC ? (plane2 + PH_NT1 - 1) / PH_NT1 : 0;
+  const long long nphi = (L.N + PH_NT1 * V - 1) / (PH_NT1 * V);
+  cudaError_t e = launch_dependent(k_phase1<S, R, ODD, XBC>, (unsigned)(nstate + nphi), PH_NT1, 0,
+                                   L.stream, a, xbc_spec(L, L.step), nstate);
+  if (e != cudaSuccess) return e;
+  const int nwall = (L.nw + PH_NT - 1) / PH_NT, nedge = XBC ? (plane2 + PH_NT - 1) / PH_NT : 0;
+  const int units = nwall + nedge + (int)((L.N + PH_NT - 1) / PH_NT);
+  const size_t smem = DIAG ? diag_thread_bytes<R>(PH_NT) : 0;
+  int grid = units;
+  if (DIAG) {
+    static int slots = 0;  // blocks resident at once (a launch shape, not a limit)
+    if (!slots) {
+      int n = 0;
+      e = resident_blocks(k_phase2<S, R, ODD, DIAG, XBC, FORCE>, PH_NT, smem, &n);
+      if (e != cudaSuccess) return e;
+      slots = n;
+    }
+    grid = units < slots ? units : slots;
+  }
+  return launch_dependent(k_phase2<S, R, ODD, DIAG, XBC, FORCE>, (unsigned)grid, PH_NT, smem,
+                          L.stream, a, nwall, nedge, units);
+}
+
+// The variant without body-force terms when F_ex = 0 (they vanish there;
+// FP64 keeps one form).
+template <class S, class R, bool ODD, bool DIAG>
+static cudaError_t launch_phases(Lattice &L, const Args<S, R> &a) {
+  if (L.bc_on) return launch_phases_f<S, R, ODD, DIAG, true, true>(L, a);
+  if constexpr (std::is_same<R, float>::value) {
+    if (a.m.Fx == R(0) && a.m.Fy == R(0) && a.m.Fz == R(0))
+      return launch_phases_f<S, R, ODD, DIAG, false, false>(L, a);
+  }
+  return launch_phases_f<S, R, ODD, DIAG, false, true>(L, a);
+}
+
 template <class S, class R, bool ODD, bool DIAG>
 static cudaError_t launch_fused_t(Lattice &L, Args<S, R> &a) {
+  if (phase_kernel_runs(L)) return launch_phases<S, R, ODD, DIAG>(L, a);
   if constexpr (pipe_storage<S>()) {
     if (pipe_eligible(L)) return launch_pipe_t<S, R, ODD, DIAG>(L, a);
   }
@@ -301,7 +373,8 @@ template <class S, class R>
 cudaError_t launch_step(Lattice &L, bool diag) {
   Args<S, R> a = make_args<S, R>(L);
   const bool odd = (L.step & 1) != 0;
-  cudaError_t e = launch_xbc<S, R>(L, a);
+  // (the two-phase step forms the boundary states itself)
+  cudaError_t e = phase_kernel_runs(L) ? cudaSuccess : launch_xbc<S, R>(L, a);
   if (e != cudaSuccess) return e;
   if (diag) {
     // Diagnostic launch d accumulates into buffer d&1 and zeroes the other.
@@ -354,9 +427,7 @@ template <class S, class R>
 void batch_build_descs(Lattice *const *lats, int n, char *host) {
   for (int l = 0; l < n; ++l) {
     for (int p = 0; p < 2; ++p) {
-      Lattice tmp = *lats[l];
-      tmp.step = p;  // selects buffers and A-A parity
-      Args<S, R> a = make_args<S, R>(tmp);
+      Args<S, R> a = make_args<S, R>(*lats[l], p);
       a.diag = lats[l]->diag + 32 * (lats[l]->ndiag & 1);
       a.diag_zero = lats[l]->diag + 32 * ((lats[l]->ndiag + 1) & 1);
       std::memcpy(host + (2 * (size_t)l + p) * sizeof(Args<S, R>), &a, sizeof a);
@@ -364,133 +435,35 @@ void batch_build_descs(Lattice *const *lats, int n, char *host) {
   }
 }
 
-template <class S, class R, bool ODD, bool DIAG, int CB = 16>
-static cudaError_t batch_pipe_attrs() {
-  static unsigned long long done = 0;  // bit d: set on device d
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const unsigned long long bit = dev < 64 ? (1ull << dev) : 0ull;
-  if (bit && (done & bit)) return cudaSuccess;
-  e = cudaFuncSetAttribute(k_batch_pipe<S, R, ODD, DIAG, CB>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)(sizeof(PipeSmem<S, R, CB>) + sizeof(Args<S, R>)));
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_batch_pipe<S, R, ODD, DIAG, CB>,
-                           cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-  if (e != cudaSuccess) return e;
-  done |= bit;
-  return cudaSuccess;
-}
-
-template <class S, class R>
-int batch_pipe_blocks_per_sm() {
-  int nb = 0;
-  if (batch_pipe_attrs<S, R, false, true>() != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-          &nb, k_batch_pipe<S, R, false, true>, PP_NT,
-          sizeof(PipeSmem<S, R>) + sizeof(Args<S, R>)) != cudaSuccess) {
-    cudaGetLastError();
-    return 1;
-  }
-  return nb > 0 ? nb : 1;
-}
-
-// One launch over the work list of one chunk size (the two lists share the
-// counter, reset before each launch on the batch stream).
-template <class S, class R, bool ODD, bool DIAG, int CB>
-static cudaError_t batch_pipe_list(const BatchDev &b, const void *items, int n) {
-  if (n == 0) return cudaSuccess;
-  cudaError_t e = batch_pipe_attrs<S, R, ODD, DIAG, CB>();
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(b.pcounter, 0, sizeof(int), b.stream);
-  if (e != cudaSuccess) return e;
-  const size_t smem = sizeof(PipeSmem<S, R, CB>) + sizeof(Args<S, R>);
-  const int grid = n < b.pgrid ? n : b.pgrid;
-  k_batch_pipe<S, R, ODD, DIAG, CB><<<grid, PP_NT, smem, b.stream>>>(
-      (const Args<S, R> *)b.descs, b.par0, (const int4 *)items, n, b.pcounter, b.bstep, b.plz);
-  return cudaGetLastError();
-}
-
-template <class S, class R, bool ODD, bool DIAG>
-static cudaError_t batch_pipe_one(const BatchDev &b) {
-  cudaError_t e = batch_pipe_list<S, R, ODD, DIAG, 16>(b, b.pitems, b.npitems);
-  if constexpr (sizeof(S) == 2) {
-    if (e == cudaSuccess) e = batch_pipe_list<S, R, ODD, DIAG, 8>(b, b.pitems8, b.npitems8);
-  }
-  return e;
-}
-
-// The pipelined lattices of a batch: their march (one launch per A-A parity
-// present at this step; tpar = parity of the batch step), then their wall
-// nodes.
-template <class S, class R>
-static cudaError_t batch_launch_pipe(const BatchDev &b, bool diag, int tpar) {
-  if (b.npitems + b.npitems8 == 0) return cudaSuccess;
+// One step of a group of lattices: both phases of all of them.
+template <class S, class R, bool XBC>
+static cudaError_t batch_launch_group(const BatchDev &b, const BatchGroup &g, int gi, bool diag,
+                                      int tpar) {
   const Args<S, R> *d = (const Args<S, R> *)b.descs;
-  cudaError_t e = cudaSuccess;
-  for (int par = 0; par < 2 && e == cudaSuccess; ++par) {
-    if (!((b.pmask >> (par ^ tpar)) & 1)) continue;  // no lattice at this parity now
-    if (par)
-      e = diag ? batch_pipe_one<S, R, true, true>(b) : batch_pipe_one<S, R, true, false>(b);
-    else
-      e = diag ? batch_pipe_one<S, R, false, true>(b) : batch_pipe_one<S, R, false, false>(b);
-  }
-  if (e != cudaSuccess || b.nwitems == 0) return e;
-  const int2 *wit = (const int2 *)b.witems;
+  const int4 *it1 = (const int4 *)b.items + g.first1, *it2 = (const int4 *)b.items + g.first2;
+  int *bstep = b.bstep + gi;
+  cudaError_t e = launch_dependent(k_batch_phase1<S, R, XBC>, (unsigned)g.n1, PH_NT1, 0, b.stream,
+                                   d, b.par0, it1, b.xspecs, bstep, tpar);
+  if (e != cudaSuccess) return e;
   if (diag)
-    k_batch_wall<S, R, true><<<b.nwitems, 128, 0, b.stream>>>(d, b.par0, wit, b.bstep);
-  else
-    k_batch_wall<S, R, false><<<b.nwitems, 128, 0, b.stream>>>(d, b.par0, wit, b.bstep);
-  return cudaGetLastError();
+    return launch_dependent(k_batch_phase2<S, R, true, XBC>, (unsigned)g.n2, PH_NT,
+                            diag_thread_bytes<R>(PH_NT), b.stream, d, b.par0, it2, bstep, tpar);
+  return launch_dependent(k_batch_phase2<S, R, false, XBC>, (unsigned)g.n2, PH_NT, 0, b.stream, d,
+                          b.par0, it2, bstep, tpar);
 }
 
 template <class S, class R>
-cudaError_t batch_launch_step(const BatchDev &b, bool diag, int tpar) {
-  cudaError_t e = cudaMemsetAsync(b.counter, 0, sizeof(int), b.stream);
-  if (e != cudaSuccess) return e;
-  const size_t smem = batch_smem<S, R>(b.bx, b.by, diag);
-  const Args<S, R> *d = (const Args<S, R> *)b.descs;
-  const int4 *it = (const int4 *)b.items;
-  if (b.nxbc > 0) {  // boundary states of the open-boundary lattices first
-    k_batch_xbc<S, R><<<dim3(b.nxbc, 32), 128, 0, b.stream>>>(d, b.par0, b.xlist, b.xspecs,
-                                                              b.bstep);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  e = batch_launch_pipe<S, R>(b, diag, tpar);
-  if (e != cudaSuccess) return e;
-  if (b.nitems == 0) {  // every lattice ran the pipelined march
-    k_batch_tick<<<1, 1, 0, b.stream>>>(b.bstep);
-    return cudaGetLastError();
-  }
-  const dim3 grid(b.grid), block(b.bx * b.by);
-  if (diag && b.nxbc > 0)
-    k_batch<S, R, true, true><<<grid, block, smem, b.stream>>>(d, b.par0, it, b.nitems, b.counter,
-                                                               b.bstep, b.bx, b.by, b.lz);
-  else if (diag)
-    k_batch<S, R, true, false><<<grid, block, smem, b.stream>>>(d, b.par0, it, b.nitems,
-                                                                b.counter, b.bstep, b.bx, b.by,
-                                                                b.lz);
-  else if (b.nxbc > 0)
-    k_batch<S, R, false, true><<<grid, block, smem, b.stream>>>(d, b.par0, it, b.nitems,
-                                                                b.counter, b.bstep, b.bx, b.by,
-                                                                b.lz);
-  else
-    k_batch<S, R, false, false><<<grid, block, smem, b.stream>>>(d, b.par0, it, b.nitems,
-                                                                 b.counter, b.bstep, b.bx, b.by,
-                                                                 b.lz);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_batch_tick<<<1, 1, 0, b.stream>>>(b.bstep);
-  return cudaGetLastError();
+cudaError_t batch_launch_step(const BatchDev &b, const BatchGroup &g, int gi, bool diag,
+                              int tpar) {
+  return g.open ? batch_launch_group<S, R, true>(b, g, gi, diag, tpar)
+                : batch_launch_group<S, R, false>(b, g, gi, diag, tpar);
 }
 
 template <class S, class R>
-int batch_max_blocks_per_sm(int bx, int by) {
+int batch_blocks_per_sm() {
   int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch<S, R, true>, bx * by,
-                                                    batch_smem<S, R>(bx, by, true)) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch_phase2<S, R, false, false>, PH_NT,
+                                                    0) != cudaSuccess) {
     cudaGetLastError();
     return 1;
   }
@@ -498,11 +471,11 @@ int batch_max_blocks_per_sm(int bx, int by) {
 }
 
 #define PFLB_INSTANTIATE(S, R)                                                   \
-  template int batch_pipe_blocks_per_sm<S, R>();                                 \
+  template int batch_blocks_per_sm<S, R>();                                      \
   template size_t batch_desc_bytes<S, R>();                                      \
   template void batch_build_descs<S, R>(Lattice *const *, int, char *);         \
-  template cudaError_t batch_launch_step<S, R>(const BatchDev &, bool, int);          \
-  template int batch_max_blocks_per_sm<S, R>(int, int);                          \
+  template cudaError_t batch_launch_step<S, R>(const BatchDev &, const BatchGroup &, int, bool, \
+                                               int);                             \
   template cudaError_t launch_init<S, R>(Lattice &, const double *, double);     \
   template cudaError_t launch_step<S, R>(Lattice &, bool);                       \
   template cudaError_t launch_macro<S, R>(Lattice &, bool);                      \

@@ -1,0 +1,346 @@
+// pflb_phase.cuh -- the step as two kernels (arXiv 2512.01032, Sec. II and
+// Sec. III A): phase 1 sums phi = sum_i h_i of every cell into the phi field
+// (and forms the boundary states of open x planes); phase 2 updates every
+// cell, its neighbours' phi read from that field.
+//
+// Against the pipelined march (pflb_pipe.cuh) this reads h twice (389 B per
+// FP32 cell instead of 305) but computes each phi once instead of once per
+// tile it touches, keeps nothing in shared memory, has no barrier, takes any
+// extent and any boundary, and hides the wall nodes' chains of loads behind
+// the bulk cells of the same launch.  Where h stays in L2 between the two
+// kernels the second read costs no DRAM traffic.  Measured (GB300, us per
+// step, against the march, or the fused kernel where that could not run):
+// FP32 drop 32^3 6.2 (10.3), 64^3 14.4 (24.7), slit 1024 x 64 x 4 20.5 (31.7)
+// before dependent launches, channel 251 x 67 x 67 88 (153); BF16 sessile
+// 128^3 121 (139).  What bounds it: at 128^3 FP32 phase 1 takes 28.7 us, the
+// copy bandwidth; phase 2 117 us, 82 % of it; below 64^3 the launches.
+//
+// A unit of work is one lane per cell: bulk cells by their linear index, wall
+// nodes by their record, boundary cells by their place in the two planes.
+#pragma once
+#include "pflb_kernels.cuh"
+#include "pflb_pipe.cuh"
+
+namespace pflb {
+
+constexpr int PH_NT1 = 128;  // threads of a phase-1 block
+// Threads of a phase-2 block: at 128 registers 8 blocks fit an SM; blocks of
+// two warps leave fewer slots idle at the end of a launch than blocks of four
+// (128^3: 116.7 against 118.8 us).
+constexpr int PH_NT = 64;
+
+// Dependent launches: a block lets the next kernel of the stream be set up
+// at once, and itself waits here until the one before has finished.
+__device__ __forceinline__ void launch_ready() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// phi of an open-boundary cell at plane x (reading R22), as xbc_cell forms it.
+template <class S, class R>
+__device__ __forceinline__ R edge_phi(const Args<S, R> &a, const XbcSpec &sp, int c, int x,
+                                      long long t) {
+  const int side = x == 0 ? 0 : 1;
+  if (sp.type[side] != 1) return (R)xbc_value(sp, side, 4, t);
+  const int ca = side ? c - 1 : c + 1;
+  if (a.flags[ca] & F_SOLID) return R(0);
+  R h[Q], s = R(0);
+  ld_h_cell<S, R>(a.hin, ca, h);
+#pragma unroll
+  for (int i = 0; i < Q; ++i) s += h[i];
+  return s;
+}
+
+// phi of the V cells from c on, summed in cell_phi's order: with V > 1 by
+// 16-byte loads (c and the number of cells are multiples of V then, so every
+// direction's address is aligned).
+template <class S, class R, bool XBC, int V>
+__device__ __forceinline__ void phase1_cells(const Args<S, R> &a, const XbcSpec &sp, int c,
+                                             long long t) {
+  R s[V];
+  uint8_t f[V];
+  if constexpr (V == 1) {
+    R h[Q];
+    f[0] = a.flags[c];
+    ld_h_cell<S, R>(a.hin, c, h);
+    s[0] = R(0);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) s[0] += h[i];
+  } else {
+    uint4 q[h_slots<S>()];
+#pragma unroll
+    for (int i = 0; i < h_slots<S>(); ++i)
+      q[i] = __ldg(reinterpret_cast<const uint4 *>(a.hin[i] + c));
+    if constexpr (V == 8) {
+      const uint2 w = *reinterpret_cast<const uint2 *>(a.flags + c);
+      memcpy(f, &w, 8);
+    } else if constexpr (V == 4) {
+      const uint32_t w = *reinterpret_cast<const uint32_t *>(a.flags + c);
+      memcpy(f, &w, 4);
+    } else {
+      const uint16_t w = *reinterpret_cast<const uint16_t *>(a.flags + c);
+      memcpy(f, &w, 2);
+    }
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      S v[V], lo[V];
+      memcpy(v, &q[i], 16);
+      if constexpr (Codec<S>::narrow) memcpy(lo, &q[Q], 16);
+#pragma unroll
+      for (int j = 0; j < V; ++j) {
+        R d = dec_pop<S, R>(v[j], i);
+        if constexpr (Codec<S>::narrow)
+          if (i == 0) d += dec_pop<S, R>(lo[j], 0);
+        s[j] = i == 0 ? d : s[j] + d;
+      }
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < V; ++j) {
+    if (f[j] & F_SOLID) s[j] = R(0);
+    if constexpr (XBC)
+      if (f[j] & F_BC) s[j] = edge_phi<S, R>(a, sp, c + j, c + j - div_by(c + j, a.dx) * a.nx, t);
+  }
+  R *out = a.phi_w + c;
+  if constexpr (V == 1) {
+    *out = s[0];
+  } else if constexpr (sizeof(R) == 8) {
+    *reinterpret_cast<double2 *>(out) = make_double2(s[0], s[1]);
+  } else {
+#pragma unroll
+    for (int j = 0; j < V; j += 4)
+      *reinterpret_cast<float4 *>(out + j) = make_float4(s[j], s[j + 1], s[j + 2], s[j + 3]);
+  }
+}
+
+// Phase 1 of cells [c0, c0 + n), by PH_NT1 threads.
+template <class S, class R, bool XBC>
+__device__ __forceinline__ void phase1_range(const Args<S, R> &a, const XbcSpec &sp, int c0, int n,
+                                             bool vec, long long t) {
+  constexpr int V = 16 / (int)sizeof(S);
+  if (vec) {
+    for (int c = c0 + (int)threadIdx.x * V; c < c0 + n; c += PH_NT1 * V)
+      phase1_cells<S, R, XBC, V>(a, sp, c, t);
+  } else {
+    for (int c = c0 + (int)threadIdx.x; c < c0 + n; c += PH_NT1)
+      phase1_cells<S, R, XBC, 1>(a, sp, c, t);
+  }
+}
+
+// Whether phase 1 may take 16 bytes per load.
+template <class S>
+__host__ __device__ inline bool phase1_vec(long long N) {
+  return N % (16 / (int)sizeof(S)) == 0;
+}
+
+// Phase 2 of wall node rec.  Everything the update reads is loaded in two
+// rounds of independent loads (the record, then what it indexes): a source
+// across a solid link is chosen by address, not by branch.  A chain of
+// conditional loads took 14 us per launch whatever the number of nodes.
+template <class S, class R, bool ODD, bool DIAG, bool XBC>
+__device__ __forceinline__ void phase2_wall(const Args<S, R> &a, int rec, DiagAcc<R> &acc) {
+  const int nw = a.nw;
+  const int c = a.wcell[rec];
+  const uint32_t lm = a.wmask[rec];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) prefetch_l1(a.wgeo + (k * nw + rec));
+  const uint8_t f = a.flags[c];
+  if constexpr (XBC)
+    if (f & F_BC) return;
+  const int z = div_by(c, a.dxy), r = c - z * (a.nx * a.ny), y = div_by(r, a.dx), x = r - y * a.nx;
+  Nbr nb;
+  nb.init(x, y, z, a.nx, a.ny, a.nz);
+  R h[Q], g[Q], val[Q];
+#pragma unroll
+  for (int i = 1; i < Q; ++i) {
+    const R *p = ((lm >> i) & 1u) ? a.ghost + ((i - 1) * nw + rec) : a.phi + (c + nb.off(i));
+    val[i] = *p;
+  }
+  ld_h_cell<S, R>(a.hin, c, h);
+#pragma unroll
+  for (int k = 0; k < Q; ++k) {
+    const S *p = ODD ? a.g[opp_of(k)] + (c + nb.off(opp_of(k))) : a.g[k] + c;
+    if (k != 0 && ((lm >> opp_of(k)) & 1u)) p = a.wp_rd + ((k - 1) * nw + rec);
+    g[k] = ld_g<S, R>(p, k);
+  }
+  R phi = R(0);
+#pragma unroll
+  for (int i = 0; i < Q; ++i) phi += h[i];
+  finish_cell<S, R, ODD, MODE_STEP, DIAG, false, COLL_X2, true>(a, x, y, z, c, f, lm, rec, nb, h,
+                                                               g, phi, val, acc);
+}
+
+// Phase 2 of boundary cell j (plane x = 0, then plane x = nx - 1).
+template <class S, class R, bool ODD>
+__device__ __forceinline__ void phase2_edge(const Args<S, R> &a, int j) {
+  const int plane = a.ny * a.nz, side = j >= plane, yz = j - side * plane;
+  const int x = side ? a.nx - 1 : 0, y = yz % a.ny, z = yz / a.ny, c = x + a.nx * yz;
+  const uint8_t f = a.flags[c];
+  if (f & F_SOLID) return;
+  Nbr nb;
+  nb.init(x, y, z, a.nx, a.ny, a.nz);
+  const int rec = (f & F_WALL) ? a.widx[c] : 0;
+  const uint32_t lm = (f & F_WALL) ? a.wmask[rec] : 0u;
+  boundary_cell<S, R, ODD, MODE_STEP>(a, x, y, z, c, lm, rec, nb);
+}
+
+// Phase 2 of bulk cell c (nothing for solid cells, wall nodes and boundary
+// cells, which have units of their own).
+template <class S, class R, bool ODD, bool DIAG, bool XBC, bool FORCE>
+__device__ __forceinline__ void phase2_bulk(const Args<S, R> &a, int c, DiagAcc<R> &acc) {
+  const uint8_t f = a.flags[c];
+  if (f & (F_SOLID | F_WALL | (XBC ? F_BC : 0))) return;
+  const int z = div_by(c, a.dxy), r = c - z * (a.nx * a.ny), y = div_by(r, a.dx), x = r - y * a.nx;
+  Nbr nb;
+  nb.init(x, y, z, a.nx, a.ny, a.nz);
+  R h[Q], g[Q], val[Q];
+  const R phi = __ldg(a.phi + c);
+#pragma unroll
+  for (int i = 1; i < Q; ++i) val[i] = __ldg(a.phi + (c + nb.off(i)));
+  gather_g<S, R, ODD>(a, c, 0u, 0, nb, g);
+  ld_h_cell<S, R>(a.hin, c, h);
+  finish_cell<S, R, ODD, MODE_STEP, DIAG, false, FORCE ? COLL_X2 : COLL_X2_NOF>(
+      a, x, y, z, c, 0, 0u, 0, nb, h, g, phi, val, acc);
+}
+
+// ------------------------------------------------------- one lattice
+// Blocks below nstate form boundary states; the others take phi cells.
+template <class S, class R, bool ODD, bool XBC>
+__global__ void __launch_bounds__(PH_NT1)
+    k_phase1(const __grid_constant__ Args<S, R> a, const __grid_constant__ XbcSpec sp, int nstate) {
+  launch_ready();
+  int b = blockIdx.x;
+  if constexpr (XBC) {
+    if (b < nstate) {
+      const int j = b * PH_NT1 + threadIdx.x;
+      if (j < 2 * a.ny * a.nz) xbc_cell<S, R, ODD>(a, sp, a.bcm, j, sp.step0);
+      return;
+    }
+    b -= nstate;
+  }
+  const bool vec = phase1_vec<S>(a.N);
+  const int per = PH_NT1 * (vec ? 16 / (int)sizeof(S) : 1), c0 = b * per;
+  phase1_range<S, R, XBC>(a, sp, c0, min(per, a.N - c0), vec, sp.step0);
+}
+
+// Units of PH_NT wall nodes, boundary cells or bulk cells, in that order (the
+// wall nodes' loads take longest).  The bulk cells are taken from the last to
+// the first: phase 1 read the last ones' h most recently, and the next phase
+// 1 begins with the h written last (144^3 FP32: 201 instead of 210 us, BF16
+// 166 instead of 172).  With diagnostics the grid is the resident
+// blocks and each takes every gridDim-th unit, so that the sums leave a block
+// once.
+template <class S, class R, bool ODD, bool DIAG, bool XBC, bool FORCE>
+__global__ void __launch_bounds__(PH_NT, sizeof(R) == 8 ? 4 : 8)
+    k_phase2(const __grid_constant__ Args<S, R> a, int nwall, int nedge, int nunits) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  R *tacc = reinterpret_cast<R *>(smem_raw);
+  __shared__ R wacc[DIAG_MAX_WARPS][32];
+  launch_ready();
+  if (DIAG) {
+    zero_next_diag(a);
+    diag_thread_zero(tacc);
+  }
+  int u = blockIdx.x;
+  do {
+    DiagAcc<R> acc;
+    acc.zero();
+    if (u < nwall) {
+      const int rec = u * PH_NT + threadIdx.x;
+      if (rec < a.nw) phase2_wall<S, R, ODD, DIAG, XBC>(a, rec, acc);
+    } else if (XBC && u < nwall + nedge) {
+      const int j = (u - nwall) * PH_NT + threadIdx.x;
+      if (j < 2 * a.ny * a.nz) phase2_edge<S, R, ODD>(a, j);
+    } else {
+      const int c = (nunits - 1 - u) * PH_NT + threadIdx.x;
+      if (c < a.N) phase2_bulk<S, R, ODD, DIAG, XBC, FORCE>(a, c, acc);
+    }
+    if (DIAG) diag_thread_add(tacc, acc);
+    u += gridDim.x;
+  } while (DIAG && u < nunits);
+  if (DIAG) diag_thread_flush(a.diag, tacc, wacc);
+}
+
+// ------------------------------------------------------ many lattices
+// Items (lattice, kind, first, count), one per block.  The block copies the
+// lattice's step descriptor for its A-A parity at this step into shared
+// memory.  A lattice's cells see exactly the arithmetic that they see in a
+// batch of their own.
+enum { PHI_CELLS = 0, PHI_STATES = 1, UPD_BULK = 2, UPD_WALL = 3, UPD_EDGE = 4 };
+
+template <class S, class R>
+__device__ __forceinline__ const Args<S, R> &batch_args(unsigned char *smem,
+                                                        const Args<S, R> *descs, int l, int p) {
+  const int *src = reinterpret_cast<const int *>(descs + 2 * l + p);
+  int *dst = reinterpret_cast<int *>(smem);
+  for (int k = threadIdx.x; k < (int)(sizeof(Args<S, R>) / 4); k += blockDim.x) dst[k] = src[k];
+  __syncthreads();
+  return *reinterpret_cast<const Args<S, R> *>(smem);
+}
+
+// tpar: parity of the batch step; bstep: batch steps since the call began
+// (boundary ramps), advanced by phase 2.
+template <class S, class R, bool XBC>
+__global__ void __launch_bounds__(PH_NT1)
+    k_batch_phase1(const Args<S, R> *__restrict__ descs, const int *__restrict__ par0,
+                   const int4 *__restrict__ items, const XbcSpec *__restrict__ specs,
+                   const int *bstep, int tpar) {
+  __shared__ __align__(16) unsigned char smem[sizeof(Args<S, R>)];
+  launch_ready();
+  const int4 it = items[blockIdx.x];
+  const int p = (par0[it.x] + tpar) & 1;
+  const Args<S, R> &a = batch_args<S, R>(smem, descs, it.x, p);
+  const XbcSpec &sp = specs[it.x];
+  const long long t = XBC ? sp.step0 + *bstep : 0;
+  if (it.y == PHI_CELLS) {
+    phase1_range<S, R, XBC>(a, sp, it.z, it.w, phase1_vec<S>(a.N), t);
+  } else if constexpr (XBC) {
+    for (int j = it.z + (int)threadIdx.x; j < it.z + it.w; j += PH_NT1) {
+      if (p)
+        xbc_cell<S, R, true>(a, sp, a.bcm, j, t);
+      else
+        xbc_cell<S, R, false>(a, sp, a.bcm, j, t);
+    }
+  }
+}
+
+template <class S, class R, bool ODD, bool DIAG, bool XBC>
+__device__ __forceinline__ void batch_update(const Args<S, R> &a, const int4 &it, R *tacc) {
+  for (int j = it.z + (int)threadIdx.x; j < it.z + it.w; j += PH_NT) {
+    DiagAcc<R> acc;
+    acc.zero();
+    if (it.y == UPD_BULK)
+      phase2_bulk<S, R, ODD, DIAG, XBC, true>(a, j, acc);
+    else if (it.y == UPD_WALL)
+      phase2_wall<S, R, ODD, DIAG, XBC>(a, j, acc);
+    else if constexpr (XBC)
+      phase2_edge<S, R, ODD>(a, j);
+    if (DIAG) diag_thread_add(tacc, acc);
+  }
+}
+
+template <class S, class R, bool DIAG, bool XBC>
+__global__ void __launch_bounds__(PH_NT, sizeof(R) == 8 ? 4 : 8)
+    k_batch_phase2(const Args<S, R> *__restrict__ descs, const int *__restrict__ par0,
+                   const int4 *__restrict__ items, int *bstep, int tpar) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  R *tacc = reinterpret_cast<R *>(smem_raw);
+  __shared__ R wacc[DIAG_MAX_WARPS][32];
+  __shared__ __align__(16) unsigned char smem[sizeof(Args<S, R>)];
+  launch_ready();
+  const int4 it = items[blockIdx.x];
+  const int p = (par0[it.x] + tpar) & 1;
+  if (DIAG) diag_thread_zero(tacc);
+  const Args<S, R> &a = batch_args<S, R>(smem, descs, it.x, p);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *bstep += 1;
+  // the first item of a lattice's bulk cells zeroes its next accumulator
+  if (DIAG && it.y == UPD_BULK && it.z == 0 && threadIdx.x < 32 && a.diag_zero)
+    a.diag_zero[threadIdx.x] = 0.0;
+  if (p)
+    batch_update<S, R, true, DIAG, XBC>(a, it, tacc);
+  else
+    batch_update<S, R, false, DIAG, XBC>(a, it, tacc);
+  if (DIAG) diag_thread_flush(a.diag, tacc, wacc);
+}
+
+}  // namespace pflb

@@ -185,10 +185,7 @@ __device__ __forceinline__ void wall_node(const Args<S, R> &a, int rec, DiagAcc<
 // ring cells of every plane it sums).  A block reads back only values it
 // wrote itself in this launch, and a cell summed by two blocks gets the
 // same bits from both (same staged h, same order), so the duplicate writes
-// are benign.  Without per-block lists (a.wl_start null) the march writes the
-// phi of its own cells in [zb, ze) that wall nodes read, for k_wall after
-// the launch.  Every thread returns with no copy in flight; the caller
-// separates two marches that reuse sm by a barrier.
+// are benign.  Every thread returns with no copy in flight.
 template <class S, class R, bool ODD, bool DIAG, bool FORCE, int CB = 16>
 __device__ __forceinline__ void pipe_march(const Args<S, R> &a, int x0, int y0, int zb, int ze,
                                            PipeSmem<S, R, CB> &sm, R (*wacc)[32], int w0 = 0,
@@ -224,10 +221,9 @@ __device__ __forceinline__ void pipe_march(const Args<S, R> &a, int x0, int y0, 
       ry = 1 + (k >> 1);
     }
   }
-  // phi field writes: 2 = own and ring cells of every summed plane (this
-  // block's wall nodes read them), 1 = own cells of [zb, ze) (k_wall or
-  // k_batch_wall reads them), 0 = none (block-uniform)
-  const int phimode = w1 > w0 ? 2 : (a.wl_start ? 0 : 1);
+  // whether this block has wall nodes, which read the phi field: own and
+  // ring cells of every summed plane go to it (block-uniform)
+  const bool phi_out = w1 > w0;
   // Plane wrap by additions: the planes touched lie within a few of [0, nz).
   auto wrapz = [nz](int zu) {
     while (zu < 0) zu += nz;
@@ -362,13 +358,13 @@ __device__ __forceinline__ void pipe_march(const Args<S, R> &a, int x0, int y0, 
     dst[(ty + 1) * PP_PW + tx + 1] = v;
     // (a column beyond a ragged edge sums the cell it wraps to, which a
     // wall node of the last valid column reads)
-    if ((f & F_NEAR) && (phimode == 2 || (phimode == 1 && valid && zu >= zb && zu < ze)))
+    if ((f & F_NEAR) && phi_out)
       a.phi_w[col + sz * wrapz(zu)] = v;
     if (ring) {
       const uint8_t fr = flag_byte(fl, ry, rx - 1);
       const R vr = (fr & F_SOLID) ? R(0) : staged_phi(st, ry, V - 1 + rx);
       dst[ry * PP_PW + rx] = vr;
-      if (phimode == 2 && (fr & F_NEAR)) a.phi_w[rcol + sz * wrapz(zu)] = vr;
+      if (phi_out && (fr & F_NEAR)) a.phi_w[rcol + sz * wrapz(zu)] = vr;
     }
   };
 
@@ -483,111 +479,6 @@ __global__ void __launch_bounds__(PP_NT, PFLB_PIPE_MIN_BLOCKS)
                                          min(zb + a.lz, a.nz),
                                          *reinterpret_cast<PipeSmem<S, R, CB> *>(smem_raw),
                                          wacc, w0, w1);
-}
-
-// Many lattices: a persistent grid pulls work items (lattice, x0, y0, z0)
-// from an atomic counter, copies the lattice's step descriptor for its A-A
-// parity at this batch step ((par0[l] + t) & 1) into shared memory and
-// marches the item's tile column over LZ planes.  The first item of each
-// lattice zeroes its next diagnostic accumulator.
-// One launch marches one parity (ODD): the items of lattices at the other
-// parity are skipped, and the host launches the second parity only when a
-// lattice of the batch is at it.  With both marches in one kernel the step
-// descriptor's fields in shared memory cost registers that k_pipe's
-// constant-bank parameters do not (168 per thread, three blocks per SM);
-// with one, the march fits k_pipe's 128 registers and four blocks per SM
-// without spilling.  CB: the staged chunk size of the items' lattices (the
-// host builds one work list per chunk size).
-template <class S, class R, bool ODD, bool DIAG, int CB = 16>
-__global__ void __launch_bounds__(PP_NT, 4)
-    k_batch_pipe(const Args<S, R> *__restrict__ descs, const int *__restrict__ par0,
-                 const int4 *__restrict__ items, int nitems, int *counter, const int *bstep,
-                 int LZ) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  PipeSmem<S, R, CB> &sm = *reinterpret_cast<PipeSmem<S, R, CB> *>(smem_raw);
-  Args<S, R> *sa = reinterpret_cast<Args<S, R> *>(smem_raw + sizeof(PipeSmem<S, R, CB>));
-  __shared__ R wacc[DIAG_MAX_WARPS][32];
-  __shared__ int s_item;
-  const int tid = threadIdx.x;
-  const int t = *bstep;
-  for (;;) {
-    if (tid == 0) s_item = atomicAdd(counter, 1);
-    __syncthreads();
-    const int idx = s_item;
-    if (idx >= nitems) break;
-    const int4 it = items[idx];
-    const int p = (par0[it.x] + t) & 1;
-    if (p != (ODD ? 1 : 0)) {  // the other parity's launch marches this item
-      __syncthreads();         // s_item is read before it is replaced
-      continue;
-    }
-    const int *src = reinterpret_cast<const int *>(descs + 2 * it.x + p);
-    int *dst = reinterpret_cast<int *>(sa);
-    for (int k = tid; k < (int)(sizeof(Args<S, R>) / 4); k += blockDim.x) dst[k] = src[k];
-    __syncthreads();
-    const Args<S, R> &a = *sa;
-    if (DIAG && it.y == 0 && it.z == 0 && it.w == 0 && tid < 32 && a.diag_zero)
-      a.diag_zero[tid] = 0.0;
-    const int ze = min(it.w + LZ, a.nz);
-    pipe_march<S, R, ODD, DIAG, true, CB>(a, it.y, it.z, it.w, ze, sm, wacc);
-    __syncthreads();  // shared descriptor and staging buffers are reused by the next item
-  }
-}
-
-// Wall nodes of a step whose bulk cells k_pipe updates, one thread per wall
-// node, launched after k_pipe on the same stream (used when the per-block
-// wall lists are not built for the launch shape in effect).  The two
-// kernels touch disjoint data: under A-A every g slot is read and written
-// by one cell, h is pushed from each cell into slots no other cell writes,
-// and only wall nodes use the ghosts and wall populations.
-template <class S, class R, bool ODD, bool DIAG>
-__global__ void __launch_bounds__(128, 4) k_wall(const __grid_constant__ Args<S, R> a) {
-  __shared__ R wacc[DIAG_MAX_WARPS][32];
-  if (DIAG) {
-    diag_block_zero(wacc);
-    __syncthreads();
-  }
-  const int rec = blockIdx.x * blockDim.x + threadIdx.x;
-  DiagAcc<R> acc;
-  acc.zero();
-  if (rec < a.nw) wall_node<S, R, ODD, DIAG>(a, rec, acc);
-  if (DIAG) {
-    diag_warp_add(wacc[threadIdx.x >> 5], acc);
-    diag_block_flush(a.diag, wacc);
-  }
-}
-
-// Wall nodes of the batch's pipelined lattices: block b takes item
-// (lattice, first record) = witems[b] and its 128 records, for the
-// lattice's parity at this batch step.
-template <class S, class R, bool DIAG>
-__global__ void __launch_bounds__(128)
-    k_batch_wall(const Args<S, R> *__restrict__ descs, const int *__restrict__ par0,
-                 const int2 *__restrict__ witems, const int *bstep) {
-  __shared__ R wacc[DIAG_MAX_WARPS][32];
-  __shared__ __align__(16) unsigned char sa_raw[sizeof(Args<S, R>)];
-  Args<S, R> *sa = reinterpret_cast<Args<S, R> *>(sa_raw);
-  const int2 it = witems[blockIdx.x];
-  const int p = (par0[it.x] + *bstep) & 1;
-  const int *src = reinterpret_cast<const int *>(descs + 2 * it.x + p);
-  int *dst = reinterpret_cast<int *>(sa);
-  for (int k = threadIdx.x; k < (int)(sizeof(Args<S, R>) / 4); k += blockDim.x) dst[k] = src[k];
-  if (DIAG) diag_block_zero(wacc);
-  __syncthreads();
-  const Args<S, R> &a = *sa;
-  const int rec = it.y + threadIdx.x;
-  DiagAcc<R> acc;
-  acc.zero();
-  if (rec < a.nw) {
-    if (p)
-      wall_node<S, R, true, DIAG>(a, rec, acc);
-    else
-      wall_node<S, R, false, DIAG>(a, rec, acc);
-  }
-  if (DIAG) {
-    diag_warp_add(wacc[threadIdx.x >> 5], acc);
-    diag_block_flush(a.diag, wacc);
-  }
 }
 
 }  // namespace pflb
