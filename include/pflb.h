@@ -68,13 +68,12 @@ enum { PFLB_FIELD_PHI = 0, PFLB_FIELD_RHO = 1, PFLB_FIELD_P = 2,
 /* Step kernels.  Every kind computes the same step; they differ in how the
  * populations reach the arithmetic:
  *   PFLB_KERNEL_PIPE (default): two kernels per step, phi of every cell
- *     and then the update, for any extent and boundaries; lattices whose h
- *     populations are larger than twice the L2 cache, with periodic x and nx
- *     a multiple of 4, run one fused z-marching kernel instead, each thread's
- *     populations of the next planes copied into shared memory one plane
- *     ahead (cp.async in 16-byte chunks; 8-byte chunks at FP16/BF16 storage
- *     when nx is not a multiple of 8), 32 x 4 tiles.  Both use the pair form
- *     of the collision;
+ *     and then the update, for any extent and boundaries; FP32 lattices whose
+ *     h populations are larger than twice the L2 cache, with periodic x, nx a
+ *     multiple of 4, few wall nodes and an extent that fills 32 x 4 tiles, run
+ *     one fused z-marching kernel instead, each thread's populations of the
+ *     next planes copied into shared memory one plane ahead (cp.async in
+ *     16-byte chunks).  Both use the pair form of the collision;
  *   PFLB_KERNEL_FUSED: one fused z-marching pass with direct loads;
  *   PFLB_KERNEL_TWOPASS: a phi pass followed by a per-cell pass;
  *   PFLB_KERNEL_FUSED_TMA: the fused pass with h staged through shared
@@ -324,8 +323,8 @@ int64_t pflb_device_bytes(const pflb_lattice *L);
 
 /* Device memory a lattice of this geometry and storage would need (bytes),
  * counted from the mask without allocating (the lazily allocated field
- * output of pflb_read and the init scratch are not included); -1 on a bad
- * argument. */
+ * output of pflb_read, the init scratch and the 48 KB of copies that the
+ * diagnostics are summed in are not included); -1 on a bad argument. */
 int64_t pflb_estimate_bytes(const pflb_geometry *geom, int storage);
 
 /* Checkpoint the full state (populations, wall buffers, ghosts, step) to a

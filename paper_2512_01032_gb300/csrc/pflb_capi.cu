@@ -121,21 +121,26 @@ size_t compute_bytes(int storage) { return storage == PFLB_STORAGE_FP64 ? 8 : 4;
 // h slots per cell: the 16-bit formats keep the rest population's remainder.
 size_t h_slots_of(int storage) { return storage_bytes(storage) == 2 ? 20 : 19; }
 
-// Whether the default kind takes the two-phase step where the pipelined march
-// could run too: up to twice the L2 cache of h populations.  Measured (us per
-// step, march / two phases): FP32 drop 64^3 24.7 / 14.4, channel 384 x 80 x 80
-// (187 MB of h) 201 / 172, drop 144^3 (227 MB) 203 / 201; beyond, drop
-// 160^3 (311 MB) 253 / 286, channel 512 x 128 x 128 (638 MB) 554 / 574; BF16
-// drop 128^3 (84 MB) 126 / 119, drop 176^3 (218 MB) 319 / 312, drop 192^3
-// (283 MB) 367 / 395.
-bool h_stays_in_l2(const Lattice *L) {
+// Whether the default kind marches the lattice (pflb_pipe.cuh): FP32 lattices
+// whose h populations are larger than twice the L2 cache, so that the two
+// phases read h twice from DRAM, with few wall nodes and an extent that fills
+// the march's 32 x 4 tiles.  us per step, march / two phases: drop 160^3 (311
+// MB of h) 255 / 275, 192^3 434 / 471, sessile 192^3 461 / 479; but drop 152^3
+// (267 MB) 239 / 235, duct 384 x 98 x 98 (280 MB, 78 % fluid) 299 / 248, channel
+// 384 x 128 x 128 (478 MB, 3.1 % wall nodes) 426 / 426, 500 x 120 x 120 (547
+// MB) 509 / 494, sessile 176^3 380 / 374.  At 16-bit storage the two phases are
+// faster throughout (drop 192^3 368 / 362, channel 380 x 130 x 130 534 / 337).
+bool march_pays(const Lattice *L) {
+  if (L->p.storage != PFLB_STORAGE_FP32) return false;
   int dev = 0, l2 = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  return (double)h_slots_of(L->p.storage) * L->N * L->elem <= 2.0 * l2;
+  const long long tiles = (long long)((L->nx + 31) / 32) * ((L->ny + 3) / 4);
+  return 19.0 * L->N * L->elem > 2.0 * l2 && L->nw < 0.025 * L->N &&
+         (double)L->nx * L->ny >= 0.9 * 128 * tiles;
 }
 
 // Planes per block in effect: the requested value, else the automatic one.
@@ -421,6 +426,7 @@ void free_all(Lattice *L) {
                   L->wcell, L->wcut, L->sfrac, L->wl, L->wl_start};
   for (void *p : ptrs)
     if (p) cudaFree(p);
+  if (L->hdiag) cudaFreeHost(L->hdiag);
   if (L->aux) cudaStreamDestroy(L->aux);
   if (L->ev_init) cudaEventDestroy(L->ev_init);
   for (cudaEvent_t &ev : L->aev)
@@ -577,8 +583,9 @@ pflb_status pflb_create(const pflb_geometry *geom, const pflb_params *params, vo
     A((void **)&L->wl, nw * sizeof(int));
     A((void **)&L->wl_start, (wall_list_blocks(L->nx, L->ny, L->nz) + 1) * sizeof(int));
   }
-  A((void **)&L->diag, 96 * sizeof(double));
+  A((void **)&L->diag, pflb::kDiagWords * sizeof(double));
   A((void **)&L->err, sizeof(int));
+  if (e == cudaSuccess) e = cudaMallocHost((void **)&L->hdiag, sizeof(pflb_diag_raw_t));
   if (e != cudaSuccess) {
     free_all(L);
     delete L;
@@ -635,7 +642,7 @@ pflb_status pflb_create(const pflb_geometry *geom, const pflb_params *params, vo
     return fail(PFLB_ERR_CUDA, std::string("upload failed: ") + cudaGetErrorString(e));
   }
   make_tmaps(L);
-  L->h_in_l2 = h_stays_in_l2(L);
+  L->march = march_pays(L);
   L->lz = resolve_lz(L);
   L->wcell_h.swap(hg.wcell);
   e = ensure_wall_lists(L, L->aux);  // nothing on the lattice's stream reads them yet
@@ -893,12 +900,9 @@ pflb_status pflb_set_diag_every(pflb_lattice *L, int every) {
   return PFLB_OK;
 }
 
-// Reads the device error flag (synchronises): a bounded wait inside a
-// kernel ran out.
-static pflb_status check_device_flag(pflb_lattice *L) {
-  int flag = 0;
-  CK(L, cudaMemcpyAsync(&flag, L->err, sizeof flag, cudaMemcpyDeviceToHost, L->stream));
-  CK(L, cudaStreamSynchronize(L->stream));
+// What a read that waited for the stream says about the device error flag: a
+// bounded wait inside a kernel ran out.
+static pflb_status device_flag_status(pflb_lattice *L, int flag) {
   if (flag) {
     L->poisoned = true;
     return fail(PFLB_ERR_TIMEOUT, "a bounded wait in the step kernel ran out; state is invalid");
@@ -937,12 +941,12 @@ static pflb_status decode_diag(const double *d, int64_t step, int nx, pflb_diag_
   return PFLB_OK;
 }
 
-static pflb_status fetch_diag(pflb_lattice *L, const double *dev, pflb_diag_t *out) {
-  double d[32];
-  CK(L, cudaMemcpyAsync(d, dev, sizeof d, cudaMemcpyDeviceToHost, L->stream));
-  pflb_status fs = check_device_flag(L);
+static pflb_status fetch_diag(pflb_lattice *L, int acc, pflb_diag_t *out) {
+  CK(L, pflb::fold_diag(*L, acc, L->step, L->hdiag));
+  CK(L, cudaStreamSynchronize(L->stream));
+  pflb_status fs = device_flag_status(L, L->hdiag->err);
   if (fs != PFLB_OK) return fs;
-  return decode_diag(d, L->step, L->nx, out);
+  return decode_diag(L->hdiag->acc, L->step, L->nx, out);
 }
 
 pflb_status pflb_last_diag_async(pflb_lattice *L, pflb_diag_raw_t *raw, int64_t *ticket) {
@@ -953,9 +957,9 @@ pflb_status pflb_last_diag_async(pflb_lattice *L, pflb_diag_raw_t *raw, int64_t 
   const int k = (int)(L->aticket % pflb::kAsyncReads);
   if (!L->aev[k]) CK(L, cudaEventCreateWithFlags(&L->aev[k], cudaEventDisableTiming));
   raw->step = L->last_diag_step;
-  CK(L, cudaMemcpyAsync(raw->acc, L->diag + 32 * ((L->ndiag - 1) & 1), sizeof raw->acc,
-                        cudaMemcpyDeviceToHost, L->stream));
-  CK(L, cudaMemcpyAsync(&raw->err, L->err, sizeof raw->err, cudaMemcpyDeviceToHost, L->stream));
+  CK(L, pflb::fold_diag(*L, (int)((L->ndiag - 1) & 1), L->last_diag_step, pflb::diag_result(*L)));
+  CK(L, cudaMemcpyAsync(raw, pflb::diag_result(*L), sizeof *raw, cudaMemcpyDeviceToHost,
+                        L->stream));
   CK(L, cudaEventRecord(L->aev[k], L->stream));
   *ticket = L->aticket++;
   return PFLB_OK;
@@ -997,7 +1001,7 @@ pflb_status pflb_last_diag(pflb_lattice *L, pflb_diag_t *out) {
   if (s != PFLB_OK) return s;
   if (!out) return fail(PFLB_ERR_ARG, "null output");
   if (L->ndiag == 0) return fail(PFLB_ERR_STATE, "no step has computed diagnostics yet");
-  pflb_status r = fetch_diag(L, L->diag + 32 * ((L->ndiag - 1) & 1), out);
+  pflb_status r = fetch_diag(L, (int)((L->ndiag - 1) & 1), out);
   out->step = L->last_diag_step;
   return r;
 }
@@ -1007,7 +1011,7 @@ pflb_status pflb_diag(pflb_lattice *L, pflb_diag_t *out) {
   if (s != PFLB_OK) return s;
   if (!out) return fail(PFLB_ERR_ARG, "null output");
   CK(L, do_macro(L, false));
-  return fetch_diag(L, L->diag + 64, out);
+  return fetch_diag(L, 2, out);
 }
 
 pflb_status pflb_read(pflb_lattice *L, int field, double *host_out) {
@@ -1024,9 +1028,11 @@ pflb_status pflb_read(pflb_lattice *L, int field, double *host_out) {
     L->dev_bytes += 6 * L->N * 8;
   }
   CK(L, do_macro(L, true));
+  CK(L, cudaMemcpyAsync(&L->hdiag->err, L->err, sizeof(int), cudaMemcpyDeviceToHost, L->stream));
   CK(L, cudaMemcpyAsync(host_out, L->out + (size_t)field * L->N, (size_t)L->N * sizeof(double),
                         cudaMemcpyDeviceToHost, L->stream));
-  return check_device_flag(L);
+  CK(L, cudaStreamSynchronize(L->stream));
+  return device_flag_status(L, L->hdiag->err);
 }
 
 int64_t pflb_get_step(const pflb_lattice *L) { return L ? L->step : -1; }
@@ -1194,7 +1200,8 @@ static pflb_status batch_build_items(pflb_batch *b) {
     }
   }
   // cells per bulk item: the launch shape's tile times its planes over 8
-  const int chunk = std::max(64, b->dev.bx * b->dev.by * b->dev.lz / 8 / 64 * 64);
+  const int chunk =
+      (int)std::min(8192LL, std::max(64LL, (long long)b->dev.bx * b->dev.by * b->dev.lz / 8 / 64 * 64));
   std::vector<int4> items;
   for (pflb::BatchGroup &g : b->groups) {
     auto add = [&](int l, int kind, int count, int per) {

@@ -13,6 +13,12 @@ namespace pflb {
 
 constexpr int kAsyncReads = 16;  // asynchronous diagnostic reads in flight per lattice
 
+// Diagnostic accumulators of a lattice: two that diagnostic steps use in turn
+// and one for the field pass, each kDiagCopies copies of 32 values, and the
+// folded record that an asynchronous read copies.
+constexpr int kDiagCopies = 64;
+constexpr size_t kDiagWords = 3 * kDiagCopies * 32 + sizeof(pflb_diag_raw_t) / sizeof(double);
+
 struct Lattice {
   int nx = 0, ny = 0, nz = 0;
   long long N = 0;
@@ -37,9 +43,10 @@ struct Lattice {
   void *sfrac = nullptr;            // [N] solid volume fraction, compute type, or null
   void *ghost = nullptr;            // [18][nw] compute type
   void *phi = nullptr;              // [N] compute type (two-pass path)
-  double *diag = nullptr;           // [32]
+  double *diag = nullptr;           // [kDiagWords]
   double *out = nullptr;            // [6][N] lazily allocated
   double *phi0 = nullptr;           // [N] init scratch, lazily allocated
+  pflb_diag_raw_t *hdiag = nullptr; // page-locked host record of synchronous reads
   int *err = nullptr;               // device error flag (bounded waits that ran out)
   CUtensorMap tmap[2];              // TMA maps of the two h buffers (staged kernel)
   bool tma_ok = false;
@@ -48,7 +55,7 @@ struct Lattice {
   int64_t last_diag_step = -1;
   int diag_every = 0;         // pflb_step accumulates diagnostics every k-th step
   int kernel = PFLB_KERNEL_PIPE;
-  bool h_in_l2 = false;       // h is small enough to stay in L2 (phase_kernel_runs)
+  bool march = false;         // the default kind marches where it can (pipe_kernel_runs)
   int bx = 32, by = 4, lz = 16;   // lz: planes per block in effect
   int lz_req = 0;                  // requested planes per block, 0 = automatic
   // open x boundaries (reading R22)
@@ -98,23 +105,22 @@ struct BatchDev {
   cudaStream_t stream = nullptr;
 };
 
-// The pipelined step kernel runs with periodic x and nx a multiple of 4 (its
-// 4-byte flag words), so that its row chunks and flag words are aligned;
-// elsewhere PFLB_KERNEL_PIPE falls back to the fused kernel.  It stages rows
-// in 16-byte chunks, or in 8-byte chunks at 16-bit storage when nx is not a
-// multiple of 8 (pipe_chunk_bytes).
+// The pipelined step kernel runs with periodic x and nx a multiple of 4, so
+// that its 16-byte row chunks and 4-byte flag words are aligned.
 inline bool pipe_layout_ok(const Lattice &L) { return !L.bc_on && L.nx % 4 == 0; }
-inline int pipe_chunk_bytes(const Lattice &L) {
-  return (L.elem == 2 && L.nx % 8 != 0) ? 8 : 16;
-}
-// The default kind runs the pipelined march on lattices whose h populations
-// do not stay in L2 between two kernels, where its layout allows it, and the
-// two-phase step on all others.
+// The default kind runs the pipelined march where it pays and its layout allows
+// it, and the two-phase step elsewhere.
 inline bool pipe_kernel_runs(const Lattice &L) {
-  return L.kernel == PFLB_KERNEL_PIPE && pipe_layout_ok(L) && !L.h_in_l2;
+  return L.kernel == PFLB_KERNEL_PIPE && L.march && pipe_layout_ok(L);
 }
 inline bool phase_kernel_runs(const Lattice &L) {
   return L.kernel == PFLB_KERNEL_PIPE && !pipe_kernel_runs(L);
+}
+
+// Accumulator of diagnostic step d (d = 2: the field pass), and the folded record.
+inline double *diag_acc(const Lattice &L, int d) { return L.diag + 32 * kDiagCopies * d; }
+inline pflb_diag_raw_t *diag_result(const Lattice &L) {
+  return reinterpret_cast<pflb_diag_raw_t *>(diag_acc(L, 3));
 }
 
 // Sets the thread-local message returned by pflb_last_error().
@@ -149,6 +155,8 @@ inline XbcSpec xbc_spec(const Lattice &L, long long step0) {
 template <class S, class R> cudaError_t launch_init(Lattice &L, const double *d_phi0, double P0);
 template <class S, class R> cudaError_t launch_step(Lattice &L, bool diag);
 template <class S, class R> cudaError_t launch_macro(Lattice &L, bool fields);
+// Queues the fold of accumulator d, with the device error flag, into out.
+cudaError_t fold_diag(Lattice &L, int d, int64_t step, pflb_diag_raw_t *out);
 template <class S, class R> cudaError_t set_model(Lattice &L);
 template <class S, class R> int max_block_threads();
 template <class S, class R> int auto_lz(const Lattice &L);

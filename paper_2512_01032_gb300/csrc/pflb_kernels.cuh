@@ -81,8 +81,9 @@ struct Args {
   const R *phi;      // [N] phi field (two-pass path and field reads)
   R *phi_w;          // the same field, written by the pipelined kernel for wall nodes' reads
   Model<R> m;
-  double *diag;      // [D_COUNT] accumulator of this launch, or null
-  double *diag_zero; // [32] accumulator of the next diagnostic launch, zeroed here
+  double *diag;      // accumulator of this launch (kDiagCopies x 32), or null
+  double *diag_zero; // accumulator of the next diagnostic launch, zeroed here
+  int reg_all;       // the diagnostic box holds every cell
   int reg[6];        // diagnostic box [x0,x1) x [y0,y1) x [z0,z1)
   double *out;       // macro outputs [6][N] (phi, rho, P, ux, uy, uz) or null
   R *bcm;            // open x boundaries: states [5][nbc] (phi, P, ux, uy, uz), or null
@@ -207,6 +208,44 @@ __device__ __forceinline__ void boundary_cell(const Args<S, R> &a, int x, int y,
   store_cell<S, R, ODD>(a, c, lm, rec, nb, h, g, val, false);
 }
 
+// Contributions of one cell to the diagnostics (a7): xp is the phi of its +x
+// neighbour.
+template <class S, class R>
+__device__ __forceinline__ void diag_cell(const Args<S, R> &a, int x, int y, int z, bool wall,
+                                          uint32_t lm, R phi, R xp, const Macro<R> &mc,
+                                          DiagAcc<R> &acc) {
+  acc.v[D_MASS] += phi;
+  if (phi >= R(0.5)) acc.v[D_NHEAVY] += R(1);
+  if (phi > R(0.95)) { acc.v[D_PH] += mc.P; acc.v[D_NPH] += R(1); }
+  if (phi < R(0.05)) { acc.v[D_PL] += mc.P; acc.v[D_NPL] += R(1); }
+  if (a.reg_all || (z >= a.reg[4] && z < a.reg[5] && x >= a.reg[0] && x < a.reg[1] &&
+                    y >= a.reg[2] && y < a.reg[3])) {
+    acc.v[D_REGION] += phi;
+    // phi = 0.5 crossings towards the +x neighbour (a fluid cell): the
+    // interface position of Sec. III C (front: phi falls through 0.5 along
+    // +x; rear: phi rises through it), linearly interpolated
+    if (!((lm >> 1) & 1u)) {
+      const R pn = xp;
+      if (phi >= R(0.5) && pn < R(0.5)) {
+        const R xc = R(x) + div_(phi - R(0.5), phi - pn);
+        acc.front = xc + R(1) > acc.front ? xc + R(1) : acc.front;
+      } else if (phi < R(0.5) && pn >= R(0.5)) {
+        const R xc = R(x) + div_(R(0.5) - phi, pn - phi);
+        acc.rear = R(a.nx) - xc > acc.rear ? R(a.nx) - xc : acc.rear;
+      }
+    }
+  }
+  if (wall && phi >= R(0.25) && phi <= R(0.75)) {
+    acc.v[D_CLN] += R(1);
+    acc.v[D_CLX] += R(x); acc.v[D_CLY] += R(y); acc.v[D_CLZ] += R(z);
+    acc.v[D_CLXX] += R(x) * R(x); acc.v[D_CLYY] += R(y) * R(y); acc.v[D_CLZZ] += R(z) * R(z);
+  }
+  const R u2 = mc.ux * mc.ux + mc.uy * mc.uy + mc.uz * mc.uz;
+  acc.v[D_KIN] += R(0.5) * mc.rho * u2;
+  if (!finite_(phi + mc.P + u2)) acc.v[D_NONFINITE] += R(1);  // NaN/Inf propagate
+  acc.umax = u2 > acc.umax ? u2 : acc.umax;  // squared; root taken at the flush
+}
+
 // Rest of the update (or macro evaluation) of one fluid cell c at (x, y, z)
 // once its populations are gathered: h[] and g[] hold the streamed
 // populations, phi = sum h, val[1..18] the phi of the 18 neighbours
@@ -307,38 +346,7 @@ __device__ __forceinline__ void finish_cell(const Args<S, R> &a, int x, int y, i
   else
     mc = macros(m, g, phi, gx, gy, gz, lap);
 
-  if (DIAG) {
-    acc.v[D_MASS] += phi;
-    if (phi >= R(0.5)) acc.v[D_NHEAVY] += R(1);
-    if (phi > R(0.95)) { acc.v[D_PH] += mc.P; acc.v[D_NPH] += R(1); }
-    if (phi < R(0.05)) { acc.v[D_PL] += mc.P; acc.v[D_NPL] += R(1); }
-    if (z >= a.reg[4] && z < a.reg[5] && x >= a.reg[0] && x < a.reg[1] && y >= a.reg[2] &&
-        y < a.reg[3]) {
-      acc.v[D_REGION] += phi;
-      // phi = 0.5 crossings towards the +x neighbour (a fluid cell): the
-      // interface position of Sec. III C (front: phi falls through 0.5 along
-      // +x; rear: phi rises through it), linearly interpolated
-      if (!((lm >> 1) & 1u)) {
-        const R pn = val[1];
-        if (phi >= R(0.5) && pn < R(0.5)) {
-          const R xc = R(x) + div_(phi - R(0.5), phi - pn);
-          acc.front = xc + R(1) > acc.front ? xc + R(1) : acc.front;
-        } else if (phi < R(0.5) && pn >= R(0.5)) {
-          const R xc = R(x) + div_(R(0.5) - phi, pn - phi);
-          acc.rear = R(a.nx) - xc > acc.rear ? R(a.nx) - xc : acc.rear;
-        }
-      }
-    }
-    if (wall && phi >= R(0.25) && phi <= R(0.75)) {
-      acc.v[D_CLN] += R(1);
-      acc.v[D_CLX] += R(x); acc.v[D_CLY] += R(y); acc.v[D_CLZ] += R(z);
-      acc.v[D_CLXX] += R(x) * R(x); acc.v[D_CLYY] += R(y) * R(y); acc.v[D_CLZZ] += R(z) * R(z);
-    }
-    const R u2 = mc.ux * mc.ux + mc.uy * mc.uy + mc.uz * mc.uz;
-    acc.v[D_KIN] += R(0.5) * mc.rho * u2;
-    if (!finite_(phi + mc.P + u2)) acc.v[D_NONFINITE] += R(1);  // NaN/Inf propagate
-    acc.umax = u2 > acc.umax ? u2 : acc.umax;  // squared; root taken at the flush
-  }
+  if (DIAG) diag_cell<S, R>(a, x, y, z, wall, lm, phi, val[1], mc, acc);
   if (MODE == MODE_MACRO) {
     if (a.out) {
       const long long N = a.N;
@@ -511,8 +519,7 @@ __device__ __forceinline__ void diag_block_flush(double *diag, R (*wacc)[32]) {
       t = is_max ? fmax(t, (double)wacc[w][k]) : t + (double)wacc[w][k];
     if (is_max) {
       // non-negative doubles order like their bit patterns; D_UMAX holds
-      // the squared speed until here
-      if (k == D_UMAX) t = sqrt(t);
+      // the squared speed until it is read
       if (t > 0.0)
         atomicMax((unsigned long long *)(diag + k), (unsigned long long)__double_as_longlong(t));
     } else if (t != 0.0) {
@@ -590,10 +597,19 @@ __device__ __forceinline__ R cell_phi(const Args<S, R> &a, int c) {
   return s;
 }
 
+// A diagnostic accumulator is kDiagCopies copies of 32 values; kernels with
+// many blocks spread their additions over the copies, k_diag_fold adds them up
+// when they are read.
+__device__ __forceinline__ double *diag_copy(double *diag) {
+  return diag + 32 * (blockIdx.x % kDiagCopies);
+}
+__device__ __forceinline__ void zero_diag(double *diag) {
+  if (diag)
+    for (int k = threadIdx.x; k < 32 * kDiagCopies; k += blockDim.x) diag[k] = 0.0;
+}
 template <class S, class R>
 __device__ __forceinline__ void zero_next_diag(const Args<S, R> &a) {
-  if (a.diag_zero && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x < 32)
-    a.diag_zero[threadIdx.x] = 0.0;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) zero_diag(a.diag_zero);
 }
 
 // --------------------------------------------------------- two-pass path

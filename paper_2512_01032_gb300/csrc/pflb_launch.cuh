@@ -78,6 +78,8 @@ static Args<S, R> make_args(const Lattice &L, int parity) {
   a.diag = nullptr;
   a.diag_zero = nullptr;
   for (int k = 0; k < 6; ++k) a.reg[k] = L.reg[k];
+  a.reg_all = L.reg[0] <= 0 && L.reg[1] >= L.nx && L.reg[2] <= 0 && L.reg[3] >= L.ny &&
+              L.reg[4] <= 0 && L.reg[5] >= L.nz;
   a.out = nullptr;
   a.bcm = L.bc_on ? (R *)L.bcm : nullptr;
   a.nbc = 2 * L.ny * L.nz;
@@ -115,7 +117,7 @@ cudaError_t launch_init(Lattice &L, const double *d_phi0, double P0) {
   L.ndiag = 0;
   L.last_diag_step = -1;
   Args<S, R> a = make_args<S, R>(L);
-  cudaError_t e = cudaMemsetAsync(L.diag, 0, 96 * sizeof(double), L.stream);
+  cudaError_t e = cudaMemsetAsync(L.diag, 0, kDiagWords * sizeof(double), L.stream);
   if (e != cudaSuccess) return e;
   const int T = 256;
   const long long B = (L.N + T - 1) / T;
@@ -153,15 +155,15 @@ static cudaError_t launch_async_t(Lattice &L, Args<float, float> &a) {
   return cudaGetLastError();
 }
 
-// The pipelined kernel (periodic x; nx a multiple of 4).
+// The pipelined kernel (FP32 storage, periodic x, nx a multiple of 4).
 template <class S>
 constexpr bool pipe_storage() {
-  return true;
+  return std::is_same<S, float>::value;
 }
 inline bool pipe_eligible(const Lattice &L) { return pipe_kernel_runs(L); }
 
 // Dynamic shared memory above 48 KB is opted into once per device.
-template <class S, class R, bool ODD, bool DIAG, bool FORCE, int CB = 16>
+template <class S, class R, bool ODD, bool DIAG, bool FORCE>
 static cudaError_t pipe_attrs() {
   static unsigned long long done = 0;  // bit d: set on device d
   int dev = 0;
@@ -169,38 +171,34 @@ static cudaError_t pipe_attrs() {
   if (e != cudaSuccess) return e;
   const unsigned long long bit = dev < 64 ? (1ull << dev) : 0ull;
   if (bit && (done & bit)) return cudaSuccess;
-  e = cudaFuncSetAttribute(k_pipe<S, R, ODD, DIAG, FORCE, CB>,
+  e = cudaFuncSetAttribute(k_pipe<S, R, ODD, DIAG, FORCE>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)sizeof(PipeSmem<S, R, CB>));
+                           (int)sizeof(PipeSmem<S, R>));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_pipe<S, R, ODD, DIAG, FORCE, CB>,
+  e = cudaFuncSetAttribute(k_pipe<S, R, ODD, DIAG, FORCE>,
                            cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   if (e != cudaSuccess) return e;
   done |= bit;
   return cudaSuccess;
 }
 
-template <class S, class R, bool ODD, bool DIAG, bool FORCE, int CB = 16>
+template <class S, class R, bool ODD, bool DIAG, bool FORCE>
 static cudaError_t launch_pipe_f(Lattice &L, Args<S, R> &a) {
-  cudaError_t e = pipe_attrs<S, R, ODD, DIAG, FORCE, CB>();
+  cudaError_t e = pipe_attrs<S, R, ODD, DIAG, FORCE>();
   if (e != cudaSuccess) return e;
   const dim3 grid((L.nx + PP_BX - 1) / PP_BX, (L.ny + PP_BY - 1) / PP_BY,
                   (L.nz + L.lz - 1) / L.lz);
   // the wall nodes of each block, listed for the planes per block in effect
   a.wl = L.nw > 0 ? L.wl : nullptr;
   a.wl_start = L.nw > 0 ? L.wl_start : nullptr;
-  k_pipe<S, R, ODD, DIAG, FORCE, CB><<<grid, PP_NT, sizeof(PipeSmem<S, R, CB>), L.stream>>>(a);
+  k_pipe<S, R, ODD, DIAG, FORCE><<<grid, PP_NT, sizeof(PipeSmem<S, R>), L.stream>>>(a);
   return cudaGetLastError();
 }
 
-// The variant without body-force terms when F_ex = 0 (they vanish there);
-// 16-bit lattices with nx = 4 mod 8 staged in 8-byte chunks.
+// The variant without body-force terms when F_ex = 0 (they vanish there).
 template <class S, class R, bool ODD, bool DIAG>
 static cudaError_t launch_pipe_t(Lattice &L, Args<S, R> &a) {
-  if constexpr (sizeof(S) == 2) {
-    if (pipe_chunk_bytes(L) == 8) return launch_pipe_f<S, R, ODD, DIAG, true, 8>(L, a);
-  }
-  if constexpr (std::is_same<R, float>::value) {  // FP64 keeps one form (parity)
+  if constexpr (std::is_same<R, float>::value) {
     if (a.m.Fx == R(0) && a.m.Fy == R(0) && a.m.Fz == R(0))
       return launch_pipe_f<S, R, ODD, DIAG, false>(L, a);
   }
@@ -225,18 +223,6 @@ static cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigne
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
-// Resident blocks of a kernel on the current device.
-template <class K>
-static cudaError_t resident_blocks(K kernel, int threads, size_t smem, int *blocks) {
-  int dev = 0, sm = 0, per = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem);
-  *blocks = sm * (per > 0 ? per : 1);
-  return e;
-}
-
 // The two-phase step of one lattice.
 template <class S, class R, bool ODD, bool DIAG, bool XBC, bool FORCE>
 static cudaError_t launch_phases_f(Lattice &L, const Args<S, R> &a) {
@@ -247,22 +233,11 @@ static cudaError_t launch_phases_f(Lattice &L, const Args<S, R> &a) {
   cudaError_t e = launch_dependent(k_phase1<S, R, ODD, XBC>, (unsigned)(nstate + nphi), PH_NT1, 0,
                                    L.stream, a, xbc_spec(L, L.step), nstate);
   if (e != cudaSuccess) return e;
-  const int nwall = (L.nw + PH_NT - 1) / PH_NT, nedge = XBC ? (plane2 + PH_NT - 1) / PH_NT : 0;
-  const int units = nwall + nedge + (int)((L.N + PH_NT - 1) / PH_NT);
-  const size_t smem = DIAG ? diag_thread_bytes<R>(PH_NT) : 0;
-  int grid = units;
-  if (DIAG) {
-    static int slots = 0;  // blocks resident at once (a launch shape, not a limit)
-    if (!slots) {
-      int n = 0;
-      e = resident_blocks(k_phase2<S, R, ODD, DIAG, XBC, FORCE>, PH_NT, smem, &n);
-      if (e != cudaSuccess) return e;
-      slots = n;
-    }
-    grid = units < slots ? units : slots;
-  }
-  return launch_dependent(k_phase2<S, R, ODD, DIAG, XBC, FORCE>, (unsigned)grid, PH_NT, smem,
-                          L.stream, a, nwall, nedge, units);
+  constexpr int NT = PH_NT;
+  const int nwall = (L.nw + NT - 1) / NT, nedge = XBC ? (plane2 + NT - 1) / NT : 0;
+  const long long grid = nwall + nedge + (L.N + NT - 1) / NT;
+  return launch_dependent(k_phase2<S, R, ODD, DIAG, XBC, FORCE>, (unsigned)grid, NT, 0, L.stream, a,
+                          nwall, nedge);
 }
 
 // The variant without body-force terms when F_ex = 0 (they vanish there;
@@ -377,9 +352,9 @@ cudaError_t launch_step(Lattice &L, bool diag) {
   cudaError_t e = phase_kernel_runs(L) ? cudaSuccess : launch_xbc<S, R>(L, a);
   if (e != cudaSuccess) return e;
   if (diag) {
-    // Diagnostic launch d accumulates into buffer d&1 and zeroes the other.
-    a.diag = L.diag + 32 * (L.ndiag & 1);
-    a.diag_zero = L.diag + 32 * ((L.ndiag + 1) & 1);
+    // Diagnostic launch d accumulates into accumulator d&1 and zeroes the other.
+    a.diag = diag_acc(L, (int)(L.ndiag & 1));
+    a.diag_zero = diag_acc(L, (int)((L.ndiag + 1) & 1));
   }
   if (L.kernel != PFLB_KERNEL_TWOPASS) {  // fused, its TMA-staged and pipelined forms
     if (odd) e = diag ? launch_fused_t<S, R, true, true>(L, a) : launch_fused_t<S, R, true, false>(L, a);
@@ -404,9 +379,9 @@ template <class S, class R>
 cudaError_t launch_macro(Lattice &L, bool fields) {
   Args<S, R> a = make_args<S, R>(L);
   a.out = fields ? L.out : nullptr;
-  a.diag = L.diag + 64;
+  a.diag = diag_acc(L, 2);
   a.diag_zero = nullptr;
-  cudaError_t e = cudaMemsetAsync(a.diag, 0, 32 * sizeof(double), L.stream);
+  cudaError_t e = cudaMemsetAsync(a.diag, 0, 32 * kDiagCopies * sizeof(double), L.stream);
   if (e == cudaSuccess) e = launch_xbc<S, R>(L, a);
   if (e != cudaSuccess) return e;
   if (L.step & 1) return launch_cell_t<S, R, true, MODE_MACRO, true>(L, a);
@@ -428,8 +403,8 @@ void batch_build_descs(Lattice *const *lats, int n, char *host) {
   for (int l = 0; l < n; ++l) {
     for (int p = 0; p < 2; ++p) {
       Args<S, R> a = make_args<S, R>(*lats[l], p);
-      a.diag = lats[l]->diag + 32 * (lats[l]->ndiag & 1);
-      a.diag_zero = lats[l]->diag + 32 * ((lats[l]->ndiag + 1) & 1);
+      a.diag = diag_acc(*lats[l], (int)(lats[l]->ndiag & 1));
+      a.diag_zero = diag_acc(*lats[l], (int)((lats[l]->ndiag + 1) & 1));
       std::memcpy(host + (2 * (size_t)l + p) * sizeof(Args<S, R>), &a, sizeof a);
     }
   }
@@ -446,8 +421,8 @@ static cudaError_t batch_launch_group(const BatchDev &b, const BatchGroup &g, in
                                    d, b.par0, it1, b.xspecs, bstep, tpar);
   if (e != cudaSuccess) return e;
   if (diag)
-    return launch_dependent(k_batch_phase2<S, R, true, XBC>, (unsigned)g.n2, PH_NT,
-                            diag_thread_bytes<R>(PH_NT), b.stream, d, b.par0, it2, bstep, tpar);
+    return launch_dependent(k_batch_phase2<S, R, true, XBC>, (unsigned)g.n2, PH_NT, 0, b.stream, d,
+                            b.par0, it2, bstep, tpar);
   return launch_dependent(k_batch_phase2<S, R, false, XBC>, (unsigned)g.n2, PH_NT, 0, b.stream, d,
                           b.par0, it2, bstep, tpar);
 }

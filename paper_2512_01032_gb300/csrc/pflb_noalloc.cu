@@ -200,7 +200,7 @@ extern "C" pflb_status pflb_fields_noalloc(int nx, int ny, int nz, const float *
   diag_out->p_heavy = d[D_NPH] > 0 ? d[D_PH] / d[D_NPH] : 0.0;
   diag_out->p_light = d[D_NPL] > 0 ? d[D_PL] / d[D_NPL] : 0.0;
   diag_out->dp = diag_out->p_heavy - diag_out->p_light;
-  diag_out->u_max = d[D_UMAX];
+  diag_out->u_max = std::sqrt(d[D_UMAX]);  // accumulated as |u|^2
   diag_out->region_mass = d[D_REGION];
   diag_out->kinetic = d[D_KIN];
   diag_out->nonfinite = d[D_NONFINITE];

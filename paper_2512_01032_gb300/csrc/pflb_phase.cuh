@@ -24,10 +24,85 @@
 namespace pflb {
 
 constexpr int PH_NT1 = 128;  // threads of a phase-1 block
-// Threads of a phase-2 block: at 128 registers 8 blocks fit an SM; blocks of
-// two warps leave fewer slots idle at the end of a launch than blocks of four
-// (128^3: 116.7 against 118.8 us).
+// Threads of a phase-2 block: blocks of two warps leave fewer slots idle at
+// the end of a launch than blocks of four (128^3: 116.7 against 118.8 us), and
+// than blocks of one (117.6 against 116.0 us BF16, 142.1 against 143.8 FP32).
 constexpr int PH_NT = 64;
+// Phase-2 blocks per SM.  With 7 a thread has 144 registers, enough for all
+// loads of a cell (19 phi, 19 g, 19 h) to be in flight at once; more warps with
+// fewer registers are slower (BF16 sessile 128^3: 7 blocks 108.7 us per step, 8
+// blocks 112.6, 9 blocks 111.6; FP32 141.8, 141.8, 150.3).
+template <class R>
+__host__ __device__ constexpr int phase2_blocks() {
+  return sizeof(R) == 8 ? 4 : 7;
+}
+
+// Diagnostic sums of one cell per lane over a warp, added to one of the copies
+// of the accumulator: eight sums by a butterfly that halves the quantities a
+// lane carries at each of its first three exchanges (9 shuffles in place of
+// 40), no shared memory and no barrier, so that the update's blocks stay
+// small.  Measured on sessile 64^3 FP32 (15 us per step without): 20.4 us with
+// sums over a block through shared memory, 28 us with resident blocks that
+// keep per-thread sums (their fixed shares of the cells wait for the wall
+// nodes).
+template <class R>
+__device__ __forceinline__ void phase_diag(double *diag, const DiagAcc<R> &d) {
+  constexpr unsigned all = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  R v[8] = {d.v[D_MASS],   d.v[D_KIN],    d.v[D_PH],  d.v[D_PL],
+            d.v[D_REGION], d.v[D_NHEAVY], d.v[D_NPH], d.v[D_NPL]};
+#pragma unroll
+  for (int half = 4; half >= 1; half >>= 1) {
+    const int o = 4 * half;  // 16, 8, 4
+    const bool hi = (lane & o) != 0;
+#pragma unroll
+    for (int j = 0; j < half; ++j) {
+      const R send = hi ? v[j] : v[j + half], keep = hi ? v[j + half] : v[j];
+      v[j] = keep + __shfl_xor_sync(all, send, o);
+    }
+  }
+  v[0] += __shfl_xor_sync(all, v[0], 2);
+  v[0] += __shfl_xor_sync(all, v[0], 1);
+  if ((lane & 3) == 0 && v[0] != R(0)) {
+    const int q = lane >> 2;  // bit 2: lane & 16, bit 1: lane & 8, bit 0: lane & 4
+    const int slot = q == 0 ? D_MASS : q == 1 ? D_KIN : q == 2 ? D_PH : q == 3 ? D_PL
+                   : q == 4 ? D_REGION : q == 5 ? D_NHEAVY : q == 6 ? D_NPH : D_NPL;
+    atomicAdd(diag + slot, (double)v[0]);
+  }
+  // largest |u|^2: non-negative, so its bits order as integers
+  if constexpr (sizeof(R) == 4) {
+    const unsigned m = __reduce_max_sync(all, __float_as_uint(d.umax));
+    if (lane == 1 && m)
+      atomicMax((unsigned long long *)(diag + D_UMAX),
+                (unsigned long long)__double_as_longlong((double)__uint_as_float(m)));
+  } else {
+    R m = d.umax;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(all, m, o));
+    if (lane == 1 && m > R(0))
+      atomicMax((unsigned long long *)(diag + D_UMAX),
+                (unsigned long long)__double_as_longlong((double)m));
+  }
+  // the rest is rare: contact line, interface crossings, non-finite values
+  if (!__any_sync(all, d.v[D_CLN] != R(0) || d.front > R(0) || d.rear > R(0) ||
+                           d.v[D_NONFINITE] != R(0)))
+    return;
+#pragma unroll
+  for (int k = D_CLN; k <= D_NONFINITE; ++k) {
+    if (k == D_KIN) continue;
+    const R s = warp_sum(d.v[k]);
+    if (lane == 0 && s != R(0)) atomicAdd(diag + k, (double)s);
+  }
+  R fr = d.front, re = d.rear;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    fr = fmax(fr, __shfl_xor_sync(all, fr, o));
+    re = fmax(re, __shfl_xor_sync(all, re, o));
+  }
+  if (lane < 2 && (lane ? re : fr) > R(0))
+    atomicMax((unsigned long long *)(diag + (lane ? D_REAR : D_FRONT)),
+              (unsigned long long)__double_as_longlong((double)(lane ? re : fr)));
+}
 
 // Dependent launches: a block lets the next kernel of the stream be set up
 // at once, and itself waits here until the one before has finished.
@@ -118,12 +193,13 @@ template <class S, class R, bool XBC>
 __device__ __forceinline__ void phase1_range(const Args<S, R> &a, const XbcSpec &sp, int c0, int n,
                                              bool vec, long long t) {
   constexpr int V = 16 / (int)sizeof(S);
+  const unsigned end = (unsigned)c0 + n;
   if (vec) {
-    for (int c = c0 + (int)threadIdx.x * V; c < c0 + n; c += PH_NT1 * V)
-      phase1_cells<S, R, XBC, V>(a, sp, c, t);
+    for (unsigned c = c0 + threadIdx.x * V; c < end; c += PH_NT1 * V)
+      phase1_cells<S, R, XBC, V>(a, sp, (int)c, t);
   } else {
-    for (int c = c0 + (int)threadIdx.x; c < c0 + n; c += PH_NT1)
-      phase1_cells<S, R, XBC, 1>(a, sp, c, t);
+    for (unsigned c = c0 + threadIdx.x; c < end; c += PH_NT1)
+      phase1_cells<S, R, XBC, 1>(a, sp, (int)c, t);
   }
 }
 
@@ -138,7 +214,7 @@ __host__ __device__ inline bool phase1_vec(long long N) {
 // across a solid link is chosen by address, not by branch.  A chain of
 // conditional loads took 14 us per launch whatever the number of nodes.
 template <class S, class R, bool ODD, bool DIAG, bool XBC>
-__device__ __forceinline__ void phase2_wall(const Args<S, R> &a, int rec, DiagAcc<R> &acc) {
+__device__ __forceinline__ void wall_update(const Args<S, R> &a, int rec, DiagAcc<R> &acc) {
   const int nw = a.nw;
   const int c = a.wcell[rec];
   const uint32_t lm = a.wmask[rec];
@@ -170,6 +246,15 @@ __device__ __forceinline__ void phase2_wall(const Args<S, R> &a, int rec, DiagAc
                                                                g, phi, val, acc);
 }
 
+// (by every lane of the warp; on: the lane has a record)
+template <class S, class R, bool ODD, bool DIAG, bool XBC>
+__device__ __forceinline__ void phase2_wall(const Args<S, R> &a, int rec, bool on) {
+  DiagAcc<R> acc;
+  acc.zero();
+  if (on) wall_update<S, R, ODD, DIAG, XBC>(a, rec, acc);
+  if (DIAG) phase_diag<R>(diag_copy(a.diag), acc);
+}
+
 // Phase 2 of boundary cell j (plane x = 0, then plane x = nx - 1).
 template <class S, class R, bool ODD>
 __device__ __forceinline__ void phase2_edge(const Args<S, R> &a, int j) {
@@ -185,22 +270,71 @@ __device__ __forceinline__ void phase2_edge(const Args<S, R> &a, int j) {
 }
 
 // Phase 2 of bulk cell c (nothing for solid cells, wall nodes and boundary
-// cells, which have units of their own).
+// cells, which have units of their own).  All loads are issued before the
+// flags decide, so that a warp waits for memory once (BF16 sessile 128^3:
+// 112.6 against 117.6 us per step).
+// Every lane of the warp calls it, those past the last cell too.
 template <class S, class R, bool ODD, bool DIAG, bool XBC, bool FORCE>
-__device__ __forceinline__ void phase2_bulk(const Args<S, R> &a, int c, DiagAcc<R> &acc) {
-  const uint8_t f = a.flags[c];
-  if (f & (F_SOLID | F_WALL | (XBC ? F_BC : 0))) return;
+__device__ __forceinline__ void phase2_bulk(const Args<S, R> &a, unsigned cell) {
+  // The diagnostics of FP32 cells are summed, by all lanes of the warp, before
+  // the collision needs the registers (sessile 128^3: 149 us per step, 157 when
+  // after it); at 16-bit storage, bound by instructions, the update is one
+  // branch and the sums come last (127 against 131 us; without diagnostics 109
+  // against 119).
+  constexpr bool MID = sizeof(S) > 2;
+  bool on = cell < (unsigned)a.N;
+  if (!MID && !DIAG && !on) return;
+  const int c = on ? (int)cell : 0;
   const int z = div_by(c, a.dxy), r = c - z * (a.nx * a.ny), y = div_by(r, a.dx), x = r - y * a.nx;
+  const Model<R> &m = a.m;
   Nbr nb;
   nb.init(x, y, z, a.nx, a.ny, a.nz);
-  R h[Q], g[Q], val[Q];
-  const R phi = __ldg(a.phi + c);
+  R h[Q], g[Q], val[Q], gx, gy, gz, lap;
+  Macro<R> mc;
+  auto load = [&] {
+    const uint8_t f = a.flags[c];
+    val[0] = __ldg(a.phi + c);
 #pragma unroll
-  for (int i = 1; i < Q; ++i) val[i] = __ldg(a.phi + (c + nb.off(i)));
-  gather_g<S, R, ODD>(a, c, 0u, 0, nb, g);
-  ld_h_cell<S, R>(a.hin, c, h);
-  finish_cell<S, R, ODD, MODE_STEP, DIAG, false, FORCE ? COLL_X2 : COLL_X2_NOF>(
-      a, x, y, z, c, 0, 0u, 0, nb, h, g, phi, val, acc);
+    for (int i = 1; i < Q; ++i) val[i] = __ldg(a.phi + (c + nb.off(i)));
+    gather_g<S, R, ODD>(a, c, 0u, 0, nb, g);
+    ld_h_cell<S, R>(a.hin, c, h);
+    return !(f & (F_SOLID | F_WALL | (XBC ? F_BC : 0)));
+  };
+  auto fields = [&] {
+    if constexpr (std::is_same<R, float>::value) {
+      cd_stencil_x2(val, gx, gy, gz, lap);
+      mc = macros_x2(m, g, val[0], gx, gy, gz, lap);
+    } else {
+      cd_stencil(val, gx, gy, gz, lap);
+      mc = macros(m, g, val[0], gx, gy, gz, lap);
+    }
+  };
+  auto update = [&] {
+    if constexpr (std::is_same<R, float>::value)
+      collide_pairs_x2<FORCE>(m, h, g, mc, val[0], gx, gy, gz, lap);
+    else
+      collide_pairs(m, h, g, mc, val[0], gx, gy, gz, lap);
+    store_cell<S, R, ODD>(a, c, 0u, 0, nb, h, g, val, false);
+  };
+  DiagAcc<R> acc;
+  acc.zero();
+  auto sums = [&] { diag_cell<S, R>(a, x, y, z, false, 0u, val[0], val[1], mc, acc); };
+  if constexpr (MID) {
+    if (on) on = load();
+    if (on) {
+      fields();
+      if (DIAG) sums();
+    }
+    if (DIAG) phase_diag<R>(diag_copy(a.diag), acc);
+    if (on) update();
+  } else {
+    if (on && load()) {
+      fields();
+      if (DIAG) sums();
+      update();
+    }
+    if (DIAG) phase_diag<R>(diag_copy(a.diag), acc);
+  }
 }
 
 // ------------------------------------------------------- one lattice
@@ -227,38 +361,23 @@ __global__ void __launch_bounds__(PH_NT1)
 // wall nodes' loads take longest).  The bulk cells are taken from the last to
 // the first: phase 1 read the last ones' h most recently, and the next phase
 // 1 begins with the h written last (144^3 FP32: 201 instead of 210 us, BF16
-// 166 instead of 172).  With diagnostics the grid is the resident
-// blocks and each takes every gridDim-th unit, so that the sums leave a block
-// once.
+// 166 instead of 172).
 template <class S, class R, bool ODD, bool DIAG, bool XBC, bool FORCE>
-__global__ void __launch_bounds__(PH_NT, sizeof(R) == 8 ? 4 : 8)
-    k_phase2(const __grid_constant__ Args<S, R> a, int nwall, int nedge, int nunits) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  R *tacc = reinterpret_cast<R *>(smem_raw);
-  __shared__ R wacc[DIAG_MAX_WARPS][32];
+__global__ void __launch_bounds__(PH_NT, phase2_blocks<R>())
+    k_phase2(const __grid_constant__ Args<S, R> a, int nwall, int nedge) {
+  constexpr int NT = PH_NT;
   launch_ready();
-  if (DIAG) {
-    zero_next_diag(a);
-    diag_thread_zero(tacc);
+  if (DIAG) zero_next_diag(a);
+  const int u = blockIdx.x;
+  if (u < nwall) {
+    const int rec = u * NT + threadIdx.x;
+    phase2_wall<S, R, ODD, DIAG, XBC>(a, rec, rec < a.nw);
+  } else if (XBC && u < nwall + nedge) {
+    const int j = (u - nwall) * NT + threadIdx.x;
+    if (j < 2 * a.ny * a.nz) phase2_edge<S, R, ODD>(a, j);
+  } else {
+    phase2_bulk<S, R, ODD, DIAG, XBC, FORCE>(a, (gridDim.x - 1 - u) * NT + threadIdx.x);
   }
-  int u = blockIdx.x;
-  do {
-    DiagAcc<R> acc;
-    acc.zero();
-    if (u < nwall) {
-      const int rec = u * PH_NT + threadIdx.x;
-      if (rec < a.nw) phase2_wall<S, R, ODD, DIAG, XBC>(a, rec, acc);
-    } else if (XBC && u < nwall + nedge) {
-      const int j = (u - nwall) * PH_NT + threadIdx.x;
-      if (j < 2 * a.ny * a.nz) phase2_edge<S, R, ODD>(a, j);
-    } else {
-      const int c = (nunits - 1 - u) * PH_NT + threadIdx.x;
-      if (c < a.N) phase2_bulk<S, R, ODD, DIAG, XBC, FORCE>(a, c, acc);
-    }
-    if (DIAG) diag_thread_add(tacc, acc);
-    u += gridDim.x;
-  } while (DIAG && u < nunits);
-  if (DIAG) diag_thread_flush(a.diag, tacc, wacc);
 }
 
 // ------------------------------------------------------ many lattices
@@ -305,42 +424,62 @@ __global__ void __launch_bounds__(PH_NT1)
 }
 
 template <class S, class R, bool ODD, bool DIAG, bool XBC>
-__device__ __forceinline__ void batch_update(const Args<S, R> &a, const int4 &it, R *tacc) {
-  for (int j = it.z + (int)threadIdx.x; j < it.z + it.w; j += PH_NT) {
-    DiagAcc<R> acc;
-    acc.zero();
+__device__ __forceinline__ void batch_update(const Args<S, R> &a, const int4 &it) {
+  for (int j0 = it.z; j0 < it.z + it.w; j0 += PH_NT) {
+    const int j = j0 + (int)threadIdx.x;
+    // (an item of bulk cells ends at the lattice's last cell or at a multiple
+    // of the block)
     if (it.y == UPD_BULK)
-      phase2_bulk<S, R, ODD, DIAG, XBC, true>(a, j, acc);
+      phase2_bulk<S, R, ODD, DIAG, XBC, true>(a, j);
     else if (it.y == UPD_WALL)
-      phase2_wall<S, R, ODD, DIAG, XBC>(a, j, acc);
-    else if constexpr (XBC)
+      phase2_wall<S, R, ODD, DIAG, XBC>(a, j, j < it.z + it.w);
+    else if (XBC && j < it.z + it.w)
       phase2_edge<S, R, ODD>(a, j);
-    if (DIAG) diag_thread_add(tacc, acc);
   }
 }
 
 template <class S, class R, bool DIAG, bool XBC>
-__global__ void __launch_bounds__(PH_NT, sizeof(R) == 8 ? 4 : 8)
+__global__ void __launch_bounds__(PH_NT, phase2_blocks<R>())
     k_batch_phase2(const Args<S, R> *__restrict__ descs, const int *__restrict__ par0,
                    const int4 *__restrict__ items, int *bstep, int tpar) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  R *tacc = reinterpret_cast<R *>(smem_raw);
-  __shared__ R wacc[DIAG_MAX_WARPS][32];
   __shared__ __align__(16) unsigned char smem[sizeof(Args<S, R>)];
   launch_ready();
   const int4 it = items[blockIdx.x];
   const int p = (par0[it.x] + tpar) & 1;
-  if (DIAG) diag_thread_zero(tacc);
   const Args<S, R> &a = batch_args<S, R>(smem, descs, it.x, p);
   if (blockIdx.x == 0 && threadIdx.x == 0) *bstep += 1;
   // the first item of a lattice's bulk cells zeroes its next accumulator
-  if (DIAG && it.y == UPD_BULK && it.z == 0 && threadIdx.x < 32 && a.diag_zero)
-    a.diag_zero[threadIdx.x] = 0.0;
+  if (DIAG && it.y == UPD_BULK && it.z == 0) zero_diag(a.diag_zero);
   if (p)
-    batch_update<S, R, true, DIAG, XBC>(a, it, tacc);
+    batch_update<S, R, true, DIAG, XBC>(a, it);
   else
-    batch_update<S, R, false, DIAG, XBC>(a, it, tacc);
-  if (DIAG) diag_thread_flush(a.diag, tacc, wacc);
+    batch_update<S, R, false, DIAG, XBC>(a, it);
+}
+
+// Sum of the copies of an accumulator and the device error flag, as the record
+// that a diagnostics read returns (256 threads).  out may be page-locked host
+// memory: a synchronous read is then this kernel and a wait, without copies.
+static __global__ void k_diag_fold(const double *__restrict__ copies, const int *err, int64_t step,
+                                   pflb_diag_raw_t *out) {
+  __shared__ double part[8][32];
+  launch_ready();
+  const int k = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double t = 0.0;
+#pragma unroll 8
+  for (int c = w; c < kDiagCopies; c += 8) {
+    const double v = copies[32 * c + k];
+    t = k >= D_UMAX ? fmax(t, v) : t + v;
+  }
+  part[w][k] = t;
+  __syncthreads();
+  if (w) return;
+  for (int j = 1; j < 8; ++j) t = k >= D_UMAX ? fmax(t, part[j][k]) : t + part[j][k];
+  out->acc[k] = k == D_UMAX ? sqrt(t) : t;  // accumulated as |u|^2
+  if (k == 0) {
+    out->step = step;
+    out->err = *err;
+    out->pad = 0;
+  }
 }
 
 }  // namespace pflb

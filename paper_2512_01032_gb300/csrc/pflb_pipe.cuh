@@ -1,7 +1,6 @@
 // pflb_pipe.cuh -- fused step kernel with asynchronous staging of the next
-// planes' populations in 16-byte chunks (8-byte chunks at 16-bit storage
-// when nx is not a multiple of 8; any storage type, periodic x, nx a
-// multiple of 4).
+// planes' populations in 16-byte chunks (FP32 storage, periodic x, nx a
+// multiple of 4; march_pays says which lattices run it).
 //
 // The step is k_fused's (arXiv 2512.01032, Sec. II and Sec. III A): one
 // thread per (x, y) column of a 32 x 4 tile marching a chunk of z planes,
@@ -31,8 +30,7 @@
 // march: each block updates the wall nodes among its cells after its last
 // plane, from a per-block list, while the SM's other blocks keep marching
 // (the wall nodes' chains of dependent loads held whole blocks at the
-// plane barriers when they were updated in the march).  16-bit storage
-// stages the stored values and decodes them when they are read.
+// plane barriers when they were updated in the march).
 //
 // Shared memory per block (FP32): h 2 planes x 19 x 6 rows x 40, g 19 x 4
 // rows x 40, flags 4 planes x 6 x 10 words, phi 4 planes x 34 x 6: 54 KB,
@@ -55,12 +53,9 @@ constexpr int PP_FW = (PP_BX + 8) / 4;        // flag words per staged row (x0 -
 #define PFLB_PIPE_MIN_BLOCKS 4
 #endif
 
-// CB: bytes per staged chunk, 16 (cp.async.cg) or 8 (cp.async.ca; 16-bit
-// storage with nx = 4 mod 8, whose odd rows start 8 bytes off a 16-byte
-// boundary).
-template <class S, class R, int CB = 16>
+template <class S, class R>
 struct alignas(16) PipeSmem {
-  static constexpr int V = CB / (int)sizeof(S);  // values per chunk
+  static constexpr int V = 16 / (int)sizeof(S);  // values per chunk
   static constexpr int W = PP_BX + 2 * V;        // staged row: x0 - V .. x0 + 32 + V
   static constexpr int NCH = W / V;              // chunks per staged row
   static constexpr int HS = h_slots<S>();        // 19, or 20 with the rest remainder
@@ -73,17 +68,6 @@ struct alignas(16) PipeSmem {
 __device__ __forceinline__ void cp_async_16(void *dst, const void *src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(dst)), "l"(src)
                : "memory");
-}
-__device__ __forceinline__ void cp_async_8(void *dst, const void *src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem_addr(dst)), "l"(src)
-               : "memory");
-}
-template <int CB>
-__device__ __forceinline__ void cp_async_chunk(void *dst, const void *src) {
-  if constexpr (CB == 16)
-    cp_async_16(dst, src);
-  else
-    cp_async_8(dst, src);
 }
 __device__ __forceinline__ void cp_async_4(void *dst, const void *src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_addr(dst)), "l"(src)
@@ -186,11 +170,11 @@ __device__ __forceinline__ void wall_node(const Args<S, R> &a, int rec, DiagAcc<
 // wrote itself in this launch, and a cell summed by two blocks gets the
 // same bits from both (same staged h, same order), so the duplicate writes
 // are benign.  Every thread returns with no copy in flight.
-template <class S, class R, bool ODD, bool DIAG, bool FORCE, int CB = 16>
+template <class S, class R, bool ODD, bool DIAG, bool FORCE>
 __device__ __forceinline__ void pipe_march(const Args<S, R> &a, int x0, int y0, int zb, int ze,
-                                           PipeSmem<S, R, CB> &sm, R (*wacc)[32], int w0 = 0,
+                                           PipeSmem<S, R> &sm, R (*wacc)[32], int w0 = 0,
                                            int w1 = 0) {
-  using SM = PipeSmem<S, R, CB>;
+  using SM = PipeSmem<S, R>;
   constexpr int V = SM::V, NCH = SM::NCH, HS = SM::HS;
   static_assert(F_SOLID == 1, "all_solid tests bit 0");
   const int tid = threadIdx.x, tx = tid % PP_BX, ty = tid / PP_BX;
@@ -288,10 +272,10 @@ __device__ __forceinline__ void pipe_march(const Args<S, R> &a, int x0, int y0, 
       const int cell = h_off[k] + zoff;
       if (!half) {
 #pragma unroll
-        for (int i = 0; i < 10; ++i) cp_async_chunk<CB>(&dst[i][r][ch * V], a.hin[i] + cell);
+        for (int i = 0; i < 10; ++i) cp_async_16(&dst[i][r][ch * V], a.hin[i] + cell);
       } else {
 #pragma unroll
-        for (int i = 10; i < HS; ++i) cp_async_chunk<CB>(&dst[i][r][ch * V], a.hin[i] + cell);
+        for (int i = 10; i < HS; ++i) cp_async_16(&dst[i][r][ch * V], a.hin[i] + cell);
       }
     }
   };
@@ -314,7 +298,7 @@ __device__ __forceinline__ void pipe_march(const Args<S, R> &a, int x0, int y0, 
         const int cell = g_off[u][1] + sz * z;
 #pragma unroll
         for (int k = 0; k < Q; ++k)
-          if (k >= k0 && k < k1) cp_async_chunk<CB>(&sm.g[k][r][ch * V], a.g[k] + cell);
+          if (k >= k0 && k < k1) cp_async_16(&sm.g[k][r][ch * V], a.g[k] + cell);
       } else {
         const int zo[3] = {sz * wrapz(zu - 1), sz * z, sz * wrapz(zu + 1)};
 #pragma unroll
@@ -325,7 +309,7 @@ __device__ __forceinline__ void pipe_march(const Args<S, R> &a, int x0, int y0, 
           const int hi = (V + PP_BX - 1 - (cxk < 0 ? cxk : 0)) / V;
           if (ch < lo || ch > hi) continue;
           // source row y - c_k and plane z - c_k
-          cp_async_chunk<CB>(&sm.g[k][r][ch * V],
+          cp_async_16(&sm.g[k][r][ch * V],
                              a.g[opp_of(k)] + (g_off[u][1 - cyk] + zo[1 - czk]));
         }
       }
@@ -456,9 +440,8 @@ __device__ __forceinline__ void pipe_march(const Args<S, R> &a, int x0, int y0, 
 }
 
 // One lattice: a grid of (tile column, chunk of lz planes) blocks.  FORCE
-// = false is the variant for a lattice without body force; CB the staged
-// chunk size (PipeSmem).
-template <class S, class R, bool ODD, bool DIAG, bool FORCE, int CB = 16>
+// = false is the variant for a lattice without body force.
+template <class S, class R, bool ODD, bool DIAG, bool FORCE>
 __global__ void __launch_bounds__(PP_NT, PFLB_PIPE_MIN_BLOCKS)
     k_pipe(const __grid_constant__ Args<S, R> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -475,9 +458,9 @@ __global__ void __launch_bounds__(PP_NT, PFLB_PIPE_MIN_BLOCKS)
     w0 = a.wl_start[b];
     w1 = a.wl_start[b + 1];
   }
-  pipe_march<S, R, ODD, DIAG, FORCE, CB>(a, blockIdx.x * PP_BX, blockIdx.y * PP_BY, zb,
+  pipe_march<S, R, ODD, DIAG, FORCE>(a, blockIdx.x * PP_BX, blockIdx.y * PP_BY, zb,
                                          min(zb + a.lz, a.nz),
-                                         *reinterpret_cast<PipeSmem<S, R, CB> *>(smem_raw),
+                                         *reinterpret_cast<PipeSmem<S, R> *>(smem_raw),
                                          wacc, w0, w1);
 }
 

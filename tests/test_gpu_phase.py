@@ -1,7 +1,7 @@
 """The default kernel's two forms against the general two-pass kernel.
 
 The default kind runs the two-phase step on most lattices and the pipelined
-march on those whose h populations are larger than twice the L2 cache; a
+march on FP32 ones whose h populations are larger than twice the L2 cache; a
 batch steps small lattices in groups and large ones by themselves.  Each form
 is compared with the two-pass kernel (pinned to the oracle by the parity
 tests) on the same inputs, at sizes where it can go wrong: cell counts that
@@ -109,9 +109,9 @@ def test_batch_of_large_small_and_open_lattices(storage):
     B.close()
 
 
-@pytest.mark.parametrize("storage,dims", [("fp32", (164, 151, 160)), ("bf16", (208, 182, 184)),
+@pytest.mark.parametrize("storage,dims", [("fp32", (160, 151, 160)), ("fp32", (188, 142, 145)),
                                           ("bf16", (204, 185, 184))])
-def test_march_of_lattices_beyond_l2(storage, dims):
+def test_lattices_beyond_l2(storage, dims):
     import torch
     h = dims[0] * dims[1] * dims[2] * (19 * 4 if storage == "fp32" else 20 * 2)
     assert h > 2 * torch.cuda.get_device_properties(0).L2_cache_size
