@@ -94,11 +94,18 @@ cudaError_t do_step(Lattice *L, bool diag) {
     return pflb::launch_step<S, R>(*L, diag);
   });
 }
-cudaError_t do_macro(Lattice *L, bool fields) {
+cudaError_t do_macro(Lattice *L) {
   return dispatch(L, [&](auto *s, auto *r) {
     using S = std::remove_pointer_t<decltype(s)>;
     using R = std::remove_pointer_t<decltype(r)>;
-    return pflb::launch_macro<S, R>(*L, fields);
+    return pflb::launch_macro<S, R>(*L);
+  });
+}
+cudaError_t do_read(Lattice *L, int field) {
+  return dispatch(L, [&](auto *s, auto *r) {
+    using S = std::remove_pointer_t<decltype(s)>;
+    using R = std::remove_pointer_t<decltype(r)>;
+    return pflb::launch_read<S, R>(*L, field);
   });
 }
 template <class F>
@@ -1010,7 +1017,7 @@ pflb_status pflb_diag(pflb_lattice *L, pflb_diag_t *out) {
   pflb_status s = check_lattice(L);
   if (s != PFLB_OK) return s;
   if (!out) return fail(PFLB_ERR_ARG, "null output");
-  CK(L, do_macro(L, false));
+  CK(L, do_macro(L));
   return fetch_diag(L, 2, out);
 }
 
@@ -1019,18 +1026,18 @@ pflb_status pflb_read(pflb_lattice *L, int field, double *host_out) {
   if (s != PFLB_OK) return s;
   if (!host_out || field < 0 || field > 5) return fail(PFLB_ERR_ARG, "bad field or output");
   if (!L->out) {
-    cudaError_t e = cudaMalloc((void **)&L->out, 6 * (size_t)L->N * sizeof(double));
+    cudaError_t e = cudaMalloc((void **)&L->out, (size_t)L->N * sizeof(double));
     if (e != cudaSuccess) {
       cudaGetLastError();
       L->out = nullptr;
       return alloc_fail(e, "device allocation failed (field output)");
     }
-    L->dev_bytes += 6 * L->N * 8;
+    L->dev_bytes += L->N * 8;
   }
-  CK(L, do_macro(L, true));
+  CK(L, do_read(L, field));
   CK(L, cudaMemcpyAsync(&L->hdiag->err, L->err, sizeof(int), cudaMemcpyDeviceToHost, L->stream));
-  CK(L, cudaMemcpyAsync(host_out, L->out + (size_t)field * L->N, (size_t)L->N * sizeof(double),
-                        cudaMemcpyDeviceToHost, L->stream));
+  CK(L, cudaMemcpyAsync(host_out, L->out, (size_t)L->N * sizeof(double), cudaMemcpyDeviceToHost,
+                        L->stream));
   CK(L, cudaStreamSynchronize(L->stream));
   return device_flag_status(L, L->hdiag->err);
 }

@@ -44,7 +44,7 @@ struct Lattice {
   void *ghost = nullptr;            // [18][nw] compute type
   void *phi = nullptr;              // [N] compute type (two-pass path)
   double *diag = nullptr;           // [kDiagWords]
-  double *out = nullptr;            // [6][N] lazily allocated
+  double *out = nullptr;            // [N] one field as doubles, lazily allocated
   double *phi0 = nullptr;           // [N] init scratch, lazily allocated
   pflb_diag_raw_t *hdiag = nullptr; // page-locked host record of synchronous reads
   int *err = nullptr;               // device error flag (bounded waits that ran out)
@@ -154,7 +154,8 @@ inline XbcSpec xbc_spec(const Lattice &L, long long step0) {
 
 template <class S, class R> cudaError_t launch_init(Lattice &L, const double *d_phi0, double P0);
 template <class S, class R> cudaError_t launch_step(Lattice &L, bool diag);
-template <class S, class R> cudaError_t launch_macro(Lattice &L, bool fields);
+template <class S, class R> cudaError_t launch_macro(Lattice &L);
+template <class S, class R> cudaError_t launch_read(Lattice &L, int field);
 // Queues the fold of accumulator d, with the device error flag, into out.
 cudaError_t fold_diag(Lattice &L, int d, int64_t step, pflb_diag_raw_t *out);
 template <class S, class R> cudaError_t set_model(Lattice &L);

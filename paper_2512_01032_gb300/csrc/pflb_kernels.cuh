@@ -85,7 +85,8 @@ struct Args {
   double *diag_zero; // accumulator of the next diagnostic launch, zeroed here
   int reg_all;       // the diagnostic box holds every cell
   int reg[6];        // diagnostic box [x0,x1) x [y0,y1) x [z0,z1)
-  double *out;       // macro outputs [6][N] (phi, rho, P, ux, uy, uz) or null
+  double *out;       // macro output [N], or null
+  int field;         // which field goes there (phi, rho, P, ux, uy, uz)
   R *bcm;            // open x boundaries: states [5][nbc] (phi, P, ux, uy, uz), or null
   int nbc;           // 2 ny nz: plane x = 0, then plane x = nx-1
   // pipelined kernel: wall records grouped by the block whose march covers
@@ -171,6 +172,12 @@ __device__ __forceinline__ void store_cell(const Args<S, R> &a, int c, uint32_t 
                                            const Nbr &nb, R h[Q], R g[Q], const R val[Q],
                                            bool in_band);
 
+// Field f (phi, rho, P, ux, uy, uz) of a cell.
+template <class R>
+__device__ __forceinline__ double field_of(int f, R phi, R rho, R P, R ux, R uy, R uz) {
+  return (double)(f == 0 ? phi : f == 1 ? rho : f == 2 ? P : f == 3 ? ux : f == 4 ? uy : uz);
+}
+
 // Open x boundary cell (reading R22): not collided; its post-collision
 // populations are the equilibria at the boundary state formed before the
 // step (k_xbc), h_i = phi_b Gamma_i(u_b), g_i = w_i P_b / T +
@@ -183,15 +190,7 @@ __device__ __forceinline__ void boundary_cell(const Args<S, R> &a, int x, int y,
   const R ux = a.bcm[2 * nb5 + j], uy = a.bcm[3 * nb5 + j], uz = a.bcm[4 * nb5 + j];
   const R rho = a.m.rho_L + phib * a.m.rho_dif;
   if (MODE == MODE_MACRO) {
-    if (a.out) {
-      const long long N = a.N;
-      a.out[c] = (double)phib;
-      a.out[N + c] = (double)rho;
-      a.out[2 * N + c] = (double)Pb;
-      a.out[3 * N + c] = (double)ux;
-      a.out[4 * N + c] = (double)uy;
-      a.out[5 * N + c] = (double)uz;
-    }
+    if (a.out) a.out[c] = field_of(a.field, phib, rho, Pb, ux, uy, uz);
     return;
   }
   const R uu15 = R(1.5) * (ux * ux + uy * uy + uz * uz);
@@ -348,15 +347,7 @@ __device__ __forceinline__ void finish_cell(const Args<S, R> &a, int x, int y, i
 
   if (DIAG) diag_cell<S, R>(a, x, y, z, wall, lm, phi, val[1], mc, acc);
   if (MODE == MODE_MACRO) {
-    if (a.out) {
-      const long long N = a.N;
-      a.out[c] = (double)phi;
-      a.out[N + c] = (double)mc.rho;
-      a.out[2 * N + c] = (double)mc.P;
-      a.out[3 * N + c] = (double)mc.ux;
-      a.out[4 * N + c] = (double)mc.uy;
-      a.out[5 * N + c] = (double)mc.uz;
-    }
+    if (a.out) a.out[c] = field_of(a.field, phi, mc.rho, mc.P, mc.ux, mc.uy, mc.uz);
     return;
   }
 
@@ -635,11 +626,6 @@ __global__ void __launch_bounds__(256) k_cell(const __grid_constant__ Args<S, R>
   acc.zero();
   if (c < a.N) {
     const uint8_t f = a.flags[c];
-    if (MODE == MODE_MACRO && (f & F_SOLID) && a.out) {
-      // fields are defined as zero on solid cells
-#pragma unroll
-      for (int k = 0; k < 6; ++k) a.out[(long long)k * a.N + c] = 0.0;
-    }
     if (!(f & F_SOLID)) {
       const int x = c % a.nx;
       const int y = (c / a.nx) % a.ny;

@@ -81,6 +81,7 @@ static Args<S, R> make_args(const Lattice &L, int parity) {
   a.reg_all = L.reg[0] <= 0 && L.reg[1] >= L.nx && L.reg[2] <= 0 && L.reg[3] >= L.ny &&
               L.reg[4] <= 0 && L.reg[5] >= L.nz;
   a.out = nullptr;
+  a.field = 0;
   a.bcm = L.bc_on ? (R *)L.bcm : nullptr;
   a.nbc = 2 * L.ny * L.nz;
   a.wl = nullptr;  // set by the pipelined launch when its lists are current
@@ -223,16 +224,22 @@ static cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigne
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+// Phase 1 of one lattice.
+template <class S, class R, bool ODD, bool XBC>
+static cudaError_t launch_phi(Lattice &L, const Args<S, R> &a) {
+  const long long V = phase1_vec<S>(L.N) ? 16 / (int)sizeof(S) : 1;
+  const int nstate = XBC ? (2 * L.ny * L.nz + PH_NT1 - 1) / PH_NT1 : 0;
+  const long long nphi = (L.N + PH_NT1 * V - 1) / (PH_NT1 * V);
+  return launch_dependent(k_phase1<S, R, ODD, XBC>, (unsigned)(nstate + nphi), PH_NT1, 0, L.stream,
+                          a, xbc_spec(L, L.step), nstate);
+}
+
 // The two-phase step of one lattice.
 template <class S, class R, bool ODD, bool DIAG, bool XBC, bool FORCE>
 static cudaError_t launch_phases_f(Lattice &L, const Args<S, R> &a) {
-  const long long V = phase1_vec<S>(L.N) ? 16 / (int)sizeof(S) : 1;
-  const int plane2 = 2 * L.ny * L.nz;
-  const int nstate = XBC ? (plane2 + PH_NT1 - 1) / PH_NT1 : 0;
-  const long long nphi = (L.N + PH_NT1 * V - 1) / (PH_NT1 * V);
-  cudaError_t e = launch_dependent(k_phase1<S, R, ODD, XBC>, (unsigned)(nstate + nphi), PH_NT1, 0,
-                                   L.stream, a, xbc_spec(L, L.step), nstate);
+  cudaError_t e = launch_phi<S, R, ODD, XBC>(L, a);
   if (e != cudaSuccess) return e;
+  const int plane2 = 2 * L.ny * L.nz;
   constexpr int NT = PH_NT;
   const int nwall = (L.nw + NT - 1) / NT, nedge = XBC ? (plane2 + NT - 1) / NT : 0;
   const long long grid = nwall + nedge + (L.N + NT - 1) / NT;
@@ -375,10 +382,10 @@ cudaError_t launch_step(Lattice &L, bool diag) {
   return e;
 }
 
+// Diagnostics of the current state.
 template <class S, class R>
-cudaError_t launch_macro(Lattice &L, bool fields) {
+cudaError_t launch_macro(Lattice &L) {
   Args<S, R> a = make_args<S, R>(L);
-  a.out = fields ? L.out : nullptr;
   a.diag = diag_acc(L, 2);
   a.diag_zero = nullptr;
   cudaError_t e = cudaMemsetAsync(a.diag, 0, 32 * kDiagCopies * sizeof(double), L.stream);
@@ -386,6 +393,35 @@ cudaError_t launch_macro(Lattice &L, bool fields) {
   if (e != cudaSuccess) return e;
   if (L.step & 1) return launch_cell_t<S, R, true, MODE_MACRO, true>(L, a);
   return launch_cell_t<S, R, false, MODE_MACRO, true>(L, a);
+}
+
+// One field of the current state into L.out.
+template <class S, class R, bool ODD, bool XBC>
+static cudaError_t launch_read_t(Lattice &L, int field) {
+  Args<S, R> a = make_args<S, R>(L);
+  a.out = L.out;
+  a.field = field;
+  if (field <= PFLB_FIELD_RHO) {
+    const long long n = L.N / (phase1_vec<S>(L.N) ? 16 / (int)sizeof(S) : 1);
+    return launch_dependent(k_read_phi<S, R, XBC>, (unsigned)((n + PH_NT1 - 1) / PH_NT1), PH_NT1, 0,
+                            L.stream, a, xbc_spec(L, L.step));
+  }
+  cudaError_t e = launch_phi<S, R, ODD, XBC>(L, a);
+  if (e != cudaSuccess) return e;
+  const int nwall = (L.nw + PH_NT - 1) / PH_NT;
+  const int nedge = XBC ? (2 * L.ny * L.nz + PH_NT - 1) / PH_NT : 0;
+  const long long grid = nwall + nedge + (L.N + PH_NT - 1) / PH_NT;
+  return launch_dependent(k_read_cell<S, R, ODD, XBC>, (unsigned)grid, PH_NT, 0, L.stream, a, nwall,
+                          nedge);
+}
+
+template <class S, class R>
+cudaError_t launch_read(Lattice &L, int field) {
+  if (L.step & 1)
+    return L.bc_on ? launch_read_t<S, R, true, true>(L, field)
+                   : launch_read_t<S, R, true, false>(L, field);
+  return L.bc_on ? launch_read_t<S, R, false, true>(L, field)
+                 : launch_read_t<S, R, false, false>(L, field);
 }
 
 template <class S, class R>
@@ -453,7 +489,8 @@ int batch_blocks_per_sm() {
                                                int);                             \
   template cudaError_t launch_init<S, R>(Lattice &, const double *, double);     \
   template cudaError_t launch_step<S, R>(Lattice &, bool);                       \
-  template cudaError_t launch_macro<S, R>(Lattice &, bool);                      \
+  template cudaError_t launch_macro<S, R>(Lattice &);                            \
+  template cudaError_t launch_read<S, R>(Lattice &, int);                        \
   template cudaError_t set_model<S, R>(Lattice &);                               \
   template int max_block_threads<S, R>();                                        \
   template int auto_lz<S, R>(const Lattice &);                                  \

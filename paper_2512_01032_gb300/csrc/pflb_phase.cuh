@@ -128,12 +128,10 @@ __device__ __forceinline__ R edge_phi(const Args<S, R> &a, const XbcSpec &sp, in
 
 // phi of the V cells from c on, summed in cell_phi's order: with V > 1 by
 // 16-byte loads (c and the number of cells are multiples of V then, so every
-// direction's address is aligned).
+// direction's address is aligned).  f returns the flags.
 template <class S, class R, bool XBC, int V>
-__device__ __forceinline__ void phase1_cells(const Args<S, R> &a, const XbcSpec &sp, int c,
-                                             long long t) {
-  R s[V];
-  uint8_t f[V];
+__device__ __forceinline__ void phi_cells(const Args<S, R> &a, const XbcSpec &sp, int c,
+                                          long long t, R s[V], uint8_t f[V]) {
   if constexpr (V == 1) {
     R h[Q];
     f[0] = a.flags[c];
@@ -176,6 +174,14 @@ __device__ __forceinline__ void phase1_cells(const Args<S, R> &a, const XbcSpec 
     if constexpr (XBC)
       if (f[j] & F_BC) s[j] = edge_phi<S, R>(a, sp, c + j, c + j - div_by(c + j, a.dx) * a.nx, t);
   }
+}
+
+template <class S, class R, bool XBC, int V>
+__device__ __forceinline__ void phase1_cells(const Args<S, R> &a, const XbcSpec &sp, int c,
+                                             long long t) {
+  R s[V];
+  uint8_t f[V];
+  phi_cells<S, R, XBC, V>(a, sp, c, t, s, f);
   R *out = a.phi_w + c;
   if constexpr (V == 1) {
     *out = s[0];
@@ -213,7 +219,7 @@ __host__ __device__ inline bool phase1_vec(long long N) {
 // rounds of independent loads (the record, then what it indexes): a source
 // across a solid link is chosen by address, not by branch.  A chain of
 // conditional loads took 14 us per launch whatever the number of nodes.
-template <class S, class R, bool ODD, bool DIAG, bool XBC>
+template <class S, class R, bool ODD, int MODE, bool DIAG, bool XBC, int PAIRS>
 __device__ __forceinline__ void wall_update(const Args<S, R> &a, int rec, DiagAcc<R> &acc) {
   const int nw = a.nw;
   const int c = a.wcell[rec];
@@ -242,8 +248,8 @@ __device__ __forceinline__ void wall_update(const Args<S, R> &a, int rec, DiagAc
   R phi = R(0);
 #pragma unroll
   for (int i = 0; i < Q; ++i) phi += h[i];
-  finish_cell<S, R, ODD, MODE_STEP, DIAG, false, COLL_X2, true>(a, x, y, z, c, f, lm, rec, nb, h,
-                                                               g, phi, val, acc);
+  finish_cell<S, R, ODD, MODE, DIAG, false, PAIRS, true>(a, x, y, z, c, f, lm, rec, nb, h, g, phi,
+                                                        val, acc);
 }
 
 // (by every lane of the warp; on: the lane has a record)
@@ -251,12 +257,12 @@ template <class S, class R, bool ODD, bool DIAG, bool XBC>
 __device__ __forceinline__ void phase2_wall(const Args<S, R> &a, int rec, bool on) {
   DiagAcc<R> acc;
   acc.zero();
-  if (on) wall_update<S, R, ODD, DIAG, XBC>(a, rec, acc);
+  if (on) wall_update<S, R, ODD, MODE_STEP, DIAG, XBC, COLL_X2>(a, rec, acc);
   if (DIAG) phase_diag<R>(diag_copy(a.diag), acc);
 }
 
 // Phase 2 of boundary cell j (plane x = 0, then plane x = nx - 1).
-template <class S, class R, bool ODD>
+template <class S, class R, bool ODD, int MODE = MODE_STEP>
 __device__ __forceinline__ void phase2_edge(const Args<S, R> &a, int j) {
   const int plane = a.ny * a.nz, side = j >= plane, yz = j - side * plane;
   const int x = side ? a.nx - 1 : 0, y = yz % a.ny, z = yz / a.ny, c = x + a.nx * yz;
@@ -266,7 +272,7 @@ __device__ __forceinline__ void phase2_edge(const Args<S, R> &a, int j) {
   nb.init(x, y, z, a.nx, a.ny, a.nz);
   const int rec = (f & F_WALL) ? a.widx[c] : 0;
   const uint32_t lm = (f & F_WALL) ? a.wmask[rec] : 0u;
-  boundary_cell<S, R, ODD, MODE_STEP>(a, x, y, z, c, lm, rec, nb);
+  boundary_cell<S, R, ODD, MODE>(a, x, y, z, c, lm, rec, nb);
 }
 
 // Phase 2 of bulk cell c (nothing for solid cells, wall nodes and boundary
@@ -377,6 +383,72 @@ __global__ void __launch_bounds__(PH_NT, phase2_blocks<R>())
     if (j < 2 * a.ny * a.nz) phase2_edge<S, R, ODD>(a, j);
   } else {
     phase2_bulk<S, R, ODD, DIAG, XBC, FORCE>(a, (gridDim.x - 1 - u) * NT + threadIdx.x);
+  }
+}
+
+// ------------------------------------------------------- field reads
+// phi or rho of every cell straight from the h populations, as doubles (zero
+// on solid cells): one pass over h, bound by its 76 + 8 bytes per FP32 cell.
+template <class S, class R, bool XBC, int V>
+__device__ __forceinline__ void read_cells(const Args<S, R> &a, const XbcSpec &sp, int c) {
+  R s[V];
+  uint8_t f[V];
+  phi_cells<S, R, XBC, V>(a, sp, c, sp.step0, s, f);
+#pragma unroll
+  for (int j = 0; j < V; ++j) {
+    const double v = (double)(a.field == 0 ? s[j] : a.m.rho_L + s[j] * a.m.rho_dif);
+    a.out[c + j] = (f[j] & F_SOLID) ? 0.0 : v;
+  }
+}
+template <class S, class R, bool XBC>
+__global__ void __launch_bounds__(PH_NT1)
+    k_read_phi(const __grid_constant__ Args<S, R> a, const __grid_constant__ XbcSpec sp) {
+  constexpr int V = 16 / (int)sizeof(S);
+  launch_ready();
+  const long long i = (long long)blockIdx.x * PH_NT1 + threadIdx.x;
+  if (phase1_vec<S>(a.N)) {
+    if (i * V < a.N) read_cells<S, R, XBC, V>(a, sp, (int)(i * V));
+  } else if (i < a.N) {
+    read_cells<S, R, XBC, 1>(a, sp, (int)i);
+  }
+}
+
+// P or a velocity component of every cell, after phase 1: the units of phase
+// 2, without the step.
+template <class S, class R, bool ODD, bool XBC>
+__global__ void __launch_bounds__(PH_NT)
+    k_read_cell(const __grid_constant__ Args<S, R> a, int nwall, int nedge) {
+  launch_ready();
+  const unsigned u = blockIdx.x;
+  if (u < (unsigned)nwall) {
+    const int rec = u * PH_NT + threadIdx.x;
+    DiagAcc<R> acc;
+    if (rec < a.nw) wall_update<S, R, ODD, MODE_MACRO, false, XBC, COLL_PLAIN>(a, rec, acc);
+  } else if (XBC && u < (unsigned)(nwall + nedge)) {
+    const int j = (u - nwall) * PH_NT + threadIdx.x;
+    if (j < 2 * a.ny * a.nz) phase2_edge<S, R, ODD, MODE_MACRO>(a, j);
+  } else {
+    const unsigned cell = (u - nwall - nedge) * PH_NT + threadIdx.x;
+    if (cell >= (unsigned)a.N) return;
+    const int c = (int)cell;
+    const uint8_t f = a.flags[c];
+    if (f & (F_WALL | (XBC ? F_BC : 0))) return;
+    if (f & F_SOLID) {
+      a.out[c] = 0.0;
+      return;
+    }
+    const int z = div_by(c, a.dxy), r = c - z * (a.nx * a.ny), y = div_by(r, a.dx),
+              x = r - y * a.nx;
+    Nbr nb;
+    nb.init(x, y, z, a.nx, a.ny, a.nz);
+    R g[Q], val[Q], gx, gy, gz, lap;
+    val[0] = __ldg(a.phi + c);
+#pragma unroll
+    for (int i = 1; i < Q; ++i) val[i] = __ldg(a.phi + (c + nb.off(i)));
+    gather_g<S, R, ODD>(a, c, 0u, 0, nb, g);
+    cd_stencil(val, gx, gy, gz, lap);
+    const Macro<R> mc = macros(a.m, g, val[0], gx, gy, gz, lap);
+    a.out[c] = field_of(a.field, val[0], mc.rho, mc.P, mc.ux, mc.uy, mc.uz);
   }
 }
 
