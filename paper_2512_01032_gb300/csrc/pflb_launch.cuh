@@ -240,22 +240,19 @@ static cudaError_t launch_phases_f(Lattice &L, const Args<S, R> &a) {
   cudaError_t e = launch_phi<S, R, ODD, XBC>(L, a);
   if (e != cudaSuccess) return e;
   const int plane2 = 2 * L.ny * L.nz;
-  constexpr int NT = PH_NT;
+  constexpr int NT = phase2_threads<R>();
   const int nwall = (L.nw + NT - 1) / NT, nedge = XBC ? (plane2 + NT - 1) / NT : 0;
   const long long grid = nwall + nedge + (L.N + NT - 1) / NT;
   return launch_dependent(k_phase2<S, R, ODD, DIAG, XBC, FORCE>, (unsigned)grid, NT, 0, L.stream, a,
                           nwall, nedge);
 }
 
-// The variant without body-force terms when F_ex = 0 (they vanish there;
-// FP64 keeps one form).
+// The variant without body-force terms when F_ex = 0 (they vanish there).
 template <class S, class R, bool ODD, bool DIAG>
 static cudaError_t launch_phases(Lattice &L, const Args<S, R> &a) {
   if (L.bc_on) return launch_phases_f<S, R, ODD, DIAG, true, true>(L, a);
-  if constexpr (std::is_same<R, float>::value) {
-    if (a.m.Fx == R(0) && a.m.Fy == R(0) && a.m.Fz == R(0))
-      return launch_phases_f<S, R, ODD, DIAG, false, false>(L, a);
-  }
+  if (a.m.Fx == R(0) && a.m.Fy == R(0) && a.m.Fz == R(0))
+    return launch_phases_f<S, R, ODD, DIAG, false, false>(L, a);
   return launch_phases_f<S, R, ODD, DIAG, false, true>(L, a);
 }
 
@@ -408,10 +405,11 @@ static cudaError_t launch_read_t(Lattice &L, int field) {
   }
   cudaError_t e = launch_phi<S, R, ODD, XBC>(L, a);
   if (e != cudaSuccess) return e;
-  const int nwall = (L.nw + PH_NT - 1) / PH_NT;
-  const int nedge = XBC ? (2 * L.ny * L.nz + PH_NT - 1) / PH_NT : 0;
-  const long long grid = nwall + nedge + (L.N + PH_NT - 1) / PH_NT;
-  return launch_dependent(k_read_cell<S, R, ODD, XBC>, (unsigned)grid, PH_NT, 0, L.stream, a, nwall,
+  constexpr int NT = phase2_threads<R>();
+  const int nwall = (L.nw + NT - 1) / NT;
+  const int nedge = XBC ? (2 * L.ny * L.nz + NT - 1) / NT : 0;
+  const long long grid = nwall + nedge + (L.N + NT - 1) / NT;
+  return launch_dependent(k_read_cell<S, R, ODD, XBC>, (unsigned)grid, NT, 0, L.stream, a, nwall,
                           nedge);
 }
 
@@ -457,9 +455,9 @@ static cudaError_t batch_launch_group(const BatchDev &b, const BatchGroup &g, in
                                    d, b.par0, it1, b.xspecs, bstep, tpar);
   if (e != cudaSuccess) return e;
   if (diag)
-    return launch_dependent(k_batch_phase2<S, R, true, XBC>, (unsigned)g.n2, PH_NT, 0, b.stream, d,
+    return launch_dependent(k_batch_phase2<S, R, true, XBC>, (unsigned)g.n2, phase2_threads<R>(), 0, b.stream, d,
                             b.par0, it2, bstep, tpar);
-  return launch_dependent(k_batch_phase2<S, R, false, XBC>, (unsigned)g.n2, PH_NT, 0, b.stream, d,
+  return launch_dependent(k_batch_phase2<S, R, false, XBC>, (unsigned)g.n2, phase2_threads<R>(), 0, b.stream, d,
                           b.par0, it2, bstep, tpar);
 }
 
@@ -473,7 +471,8 @@ cudaError_t batch_launch_step(const BatchDev &b, const BatchGroup &g, int gi, bo
 template <class S, class R>
 int batch_blocks_per_sm() {
   int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch_phase2<S, R, false, false>, PH_NT,
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch_phase2<S, R, false, false>,
+                                                    phase2_threads<R>(),
                                                     0) != cudaSuccess) {
     cudaGetLastError();
     return 1;

@@ -27,14 +27,19 @@ constexpr int PH_NT1 = 128;  // threads of a phase-1 block
 // Threads of a phase-2 block: blocks of two warps leave fewer slots idle at
 // the end of a launch than blocks of four (128^3: 116.7 against 118.8 us), and
 // than blocks of one (117.6 against 116.0 us BF16, 142.1 against 143.8 FP32).
-constexpr int PH_NT = 64;
+// At FP64 an SM issues one warp's operation in 16 clocks, so the warps per SM
+// should be even: blocks of one.
+template <class R>
+__host__ __device__ constexpr int phase2_threads() {
+  return sizeof(R) == 8 ? 32 : 64;
+}
 // Phase-2 blocks per SM.  With 7 a thread has 144 registers, enough for all
 // loads of a cell (19 phi, 19 g, 19 h) to be in flight at once; more warps with
 // fewer registers are slower (BF16 sessile 128^3: 7 blocks 108.7 us per step, 8
 // blocks 112.6, 9 blocks 111.6; FP32 141.8, 141.8, 150.3).
 template <class R>
 __host__ __device__ constexpr int phase2_blocks() {
-  return sizeof(R) == 8 ? 4 : 7;
+  return sizeof(R) == 8 ? 8 : 7;
 }
 
 // Diagnostic sums of one cell per lane over a warp, added to one of the copies
@@ -319,7 +324,7 @@ __device__ __forceinline__ void phase2_bulk(const Args<S, R> &a, unsigned cell) 
     if constexpr (std::is_same<R, float>::value)
       collide_pairs_x2<FORCE>(m, h, g, mc, val[0], gx, gy, gz, lap);
     else
-      collide_pairs(m, h, g, mc, val[0], gx, gy, gz, lap);
+      collide_pairs_lean<R, FORCE>(m, h, g, mc, val[0], gx, gy, gz, lap);
     store_cell<S, R, ODD>(a, c, 0u, 0, nb, h, g, val, false);
   };
   DiagAcc<R> acc;
@@ -363,15 +368,15 @@ __global__ void __launch_bounds__(PH_NT1)
   phase1_range<S, R, XBC>(a, sp, c0, min(per, a.N - c0), vec, sp.step0);
 }
 
-// Units of PH_NT wall nodes, boundary cells or bulk cells, in that order (the
+// Blocks of wall nodes, boundary cells or bulk cells, in that order (the
 // wall nodes' loads take longest).  The bulk cells are taken from the last to
 // the first: phase 1 read the last ones' h most recently, and the next phase
 // 1 begins with the h written last (144^3 FP32: 201 instead of 210 us, BF16
 // 166 instead of 172).
 template <class S, class R, bool ODD, bool DIAG, bool XBC, bool FORCE>
-__global__ void __launch_bounds__(PH_NT, phase2_blocks<R>())
+__global__ void __launch_bounds__(phase2_threads<R>(), phase2_blocks<R>())
     k_phase2(const __grid_constant__ Args<S, R> a, int nwall, int nedge) {
-  constexpr int NT = PH_NT;
+  constexpr int NT = phase2_threads<R>();
   launch_ready();
   if (DIAG) zero_next_diag(a);
   const int u = blockIdx.x;
@@ -416,19 +421,20 @@ __global__ void __launch_bounds__(PH_NT1)
 // P or a velocity component of every cell, after phase 1: the units of phase
 // 2, without the step.
 template <class S, class R, bool ODD, bool XBC>
-__global__ void __launch_bounds__(PH_NT)
+__global__ void __launch_bounds__(phase2_threads<R>())
     k_read_cell(const __grid_constant__ Args<S, R> a, int nwall, int nedge) {
+  constexpr int NT = phase2_threads<R>();
   launch_ready();
   const unsigned u = blockIdx.x;
   if (u < (unsigned)nwall) {
-    const int rec = u * PH_NT + threadIdx.x;
+    const int rec = u * NT + threadIdx.x;
     DiagAcc<R> acc;
     if (rec < a.nw) wall_update<S, R, ODD, MODE_MACRO, false, XBC, COLL_PLAIN>(a, rec, acc);
   } else if (XBC && u < (unsigned)(nwall + nedge)) {
-    const int j = (u - nwall) * PH_NT + threadIdx.x;
+    const int j = (u - nwall) * NT + threadIdx.x;
     if (j < 2 * a.ny * a.nz) phase2_edge<S, R, ODD, MODE_MACRO>(a, j);
   } else {
-    const unsigned cell = (u - nwall - nedge) * PH_NT + threadIdx.x;
+    const unsigned cell = (u - nwall - nedge) * NT + threadIdx.x;
     if (cell >= (unsigned)a.N) return;
     const int c = (int)cell;
     const uint8_t f = a.flags[c];
@@ -497,7 +503,7 @@ __global__ void __launch_bounds__(PH_NT1)
 
 template <class S, class R, bool ODD, bool DIAG, bool XBC>
 __device__ __forceinline__ void batch_update(const Args<S, R> &a, const int4 &it) {
-  for (int j0 = it.z; j0 < it.z + it.w; j0 += PH_NT) {
+  for (int j0 = it.z; j0 < it.z + it.w; j0 += phase2_threads<R>()) {
     const int j = j0 + (int)threadIdx.x;
     // (an item of bulk cells ends at the lattice's last cell or at a multiple
     // of the block)
@@ -511,7 +517,7 @@ __device__ __forceinline__ void batch_update(const Args<S, R> &a, const int4 &it
 }
 
 template <class S, class R, bool DIAG, bool XBC>
-__global__ void __launch_bounds__(PH_NT, phase2_blocks<R>())
+__global__ void __launch_bounds__(phase2_threads<R>(), phase2_blocks<R>())
     k_batch_phase2(const Args<S, R> *__restrict__ descs, const int *__restrict__ par0,
                    const int4 *__restrict__ items, int *bstep, int tpar) {
   __shared__ __align__(16) unsigned char smem[sizeof(Args<S, R>)];
