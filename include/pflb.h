@@ -371,7 +371,7 @@ pflb_status pflb_fields_noalloc(int nx, int ny, int nz, const float *h_dev, cons
 
 /* ------------------------------------------------------------- batches
  * Many independent lattices (of any sizes) advanced together.  Lattices of
- * less than 400000 cells are put into groups of up to 600000 cells, each
+ * less than 131072 cells are put into groups of up to 600000 cells, each
  * stepped by the two kernels of the default kind over one work list, one item
  * per block (a range of one lattice's cells, wall nodes or boundary cells), so
  * that small lattices that could not fill the GPU on their own share it and a
@@ -389,7 +389,7 @@ typedef struct pflb_batch pflb_batch;
 pflb_status pflb_batch_create(pflb_lattice *const *lattices, int count, void *cuda_stream,
                               pflb_batch **out);
 
-/* Launch shape of the groups: a work item of bulk cells holds bx * by * lz / 8
+/* Launch shape of the groups: a work item of bulk cells holds bx * by * lz / 16
  * of them (bx and by under the rules of pflb_set_kernel); zeros keep the
  * current values (default 32 x 4 x 16).  blocks_per_sm is accepted (>= 0) and
  * bounds the value that pflb_batch_tune reports; the grids hold one block per

@@ -167,7 +167,7 @@ int resolve_lz(Lattice *L) {
 // stream once created, so that steps queued before use the previous lists);
 // copies from pageable memory have read the host vectors on return.
 cudaError_t ensure_wall_lists(Lattice *L, cudaStream_t st) {
-  if (!L->wl || L->nw == 0 || L->wl_lz == L->lz || !pflb::pipe_layout_ok(*L)) return cudaSuccess;
+  if (!L->wl || L->nw == 0 || L->wl_lz == L->lz || !pflb::pipe_kernel_runs(*L)) return cudaSuccess;
   const int lz = L->lz, gx = (L->nx + 31) / 32, gy = (L->ny + 3) / 4;
   const int nch = (L->nz + lz - 1) / lz;
   const size_t nb = (size_t)gx * gy * nch;
@@ -1167,9 +1167,12 @@ static pflb_status batch_fail(pflb_batch *b, cudaError_t e, const char *what) {
     if (e_ != cudaSuccess) return batch_fail(b, e_, #call);  \
   } while (0)
 
-// A lattice of this many cells or more fills the GPU by itself: it is
-// stepped by its own kernels, all steps of a call in a row.
-static constexpr long long kAloneCells = 400000;
+// A lattice of this many cells or more is stepped by its own kernels, all
+// steps of a call in a row.  us per step and lattice, own kernels / in a group
+// of twelve: 32^3 FP32 9.6 / 3.1, 48^3 11.0 / 10.5, 56^3 12.6 / 16.7 (BF16 12.8 /
+// 12.7), 72^3 22.6 / 33 (a group's blocks read their lattice's descriptor from
+// shared memory).
+static constexpr long long kAloneCells = 131072;
 // Cells of a group of smaller ones: enough to fill the GPU, few enough that
 // their state stays in L2 from step to step.
 static constexpr long long kGroupCells = 600000;
@@ -1206,9 +1209,9 @@ static pflb_status batch_build_items(pflb_batch *b) {
       cells += L->N;
     }
   }
-  // cells per bulk item: the launch shape's tile times its planes over 8
+  // cells per bulk item: the launch shape's tile times its planes over 16
   const int chunk =
-      (int)std::min(8192LL, std::max(64LL, (long long)b->dev.bx * b->dev.by * b->dev.lz / 8 / 64 * 64));
+      (int)std::min(8192LL, std::max(64LL, (long long)b->dev.bx * b->dev.by * b->dev.lz / 16 / 64 * 64));
   std::vector<int4> items;
   for (pflb::BatchGroup &g : b->groups) {
     auto add = [&](int l, int kind, int count, int per) {

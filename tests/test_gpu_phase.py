@@ -83,7 +83,7 @@ def test_two_phase_step_matches_two_pass(dims, walls, bounds, storage):
 
 @pytest.mark.parametrize("storage", ["fp32", "bf16"])
 def test_batch_of_large_small_and_open_lattices(storage):
-    """Lattices of 400000 cells and more are stepped by themselves inside a
+    """Lattices of 131072 cells and more are stepped by themselves inside a
     batch: the same bits as outside it.  Small and open ones, stepped in
     groups, agree with the two-pass kernel."""
     from paper_2512_01032_gb300 import pflb
