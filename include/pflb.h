@@ -73,7 +73,9 @@ enum { PFLB_FIELD_PHI = 0, PFLB_FIELD_RHO = 1, PFLB_FIELD_P = 2,
  *     multiple of 4, few wall nodes and an extent that fills 32 x 4 tiles, run
  *     one fused z-marching kernel instead, each thread's populations of the
  *     next planes copied into shared memory one plane ahead (cp.async in
- *     16-byte chunks).  Both use the pair form of the collision;
+ *     16-byte chunks).  Both use the pair form of the collision, but for
+ *     FP32 lattices with open x boundaries or nx not a multiple of 4, which
+ *     take it per direction as PFLB_KERNEL_FUSED does;
  *   PFLB_KERNEL_FUSED: one fused z-marching pass with direct loads;
  *   PFLB_KERNEL_TWOPASS: a phi pass followed by a per-cell pass;
  *   PFLB_KERNEL_FUSED_TMA: the fused pass with h staged through shared
@@ -420,8 +422,8 @@ void pflb_batch_destroy(pflb_batch *b);
  * queued requests in arrival order while their estimated device footprint
  * (pflb_estimate_bytes) fits the HBM budget (and the optional caps on
  * resident requests and cells), advances every resident request by
- * steps_per_tick steps (one persistent batch kernel per step, or one launch
- * per request in plain mode), checks each request's diagnostics once, and
+ * steps_per_tick steps (one batch call, or one step call per request in
+ * plain mode), checks each request's diagnostics once, and
  * retires the finished ones, freeing their memory.  Admission's host work
  * (building and uploading a new lattice) runs while the tick's steps run on
  * the GPU; admitted requests start at the next tick.
@@ -435,7 +437,7 @@ typedef struct {
   int storage;             /* population storage of every request (PFLB_STORAGE_*) */
   int steps_per_tick;      /* steps between breakthrough checks (>= 1) */
   int max_active;          /* resident request cap, 0 = budget only */
-  int batched;             /* 1: one batch kernel per step; 0: one launch per request */
+  int batched;             /* 1: one batch call per tick; 0: one step call per request */
   int64_t max_active_cells;/* cap on the summed cells of resident requests, 0 = none (a
                               request larger than the cap still runs when it is alone) */
 } pflb_server_config;

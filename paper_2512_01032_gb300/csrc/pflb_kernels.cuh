@@ -65,6 +65,7 @@ struct Args {
   int N;
   int nw;
   FastDiv dx, dxy;       // by nx and by nx ny
+  int plain;             // nx not a multiple of 4 (open_form)
   const S *hin[Q + 1];   // direction bases of the h buffer being read (+ rest remainder)
   S *hout[Q + 1];        // direction bases of the h buffer being written
   S *g[Q];           // direction bases of the g buffer (in place)

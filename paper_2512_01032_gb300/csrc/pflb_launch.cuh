@@ -55,6 +55,7 @@ static Args<S, R> make_args(const Lattice &L, int parity) {
   a.nw = L.nw;
   a.dx = fast_div((uint32_t)L.nx);
   a.dxy = fast_div((uint32_t)L.nx * (uint32_t)L.ny);
+  a.plain = L.nx % 4 != 0;
   const int rd = parity;
   for (int i = 0; i < Q + 1; ++i) {
     const bool have = i < h_slots<S>();
@@ -235,7 +236,7 @@ static cudaError_t launch_phi(Lattice &L, const Args<S, R> &a) {
 }
 
 // The two-phase step of one lattice.
-template <class S, class R, bool ODD, bool DIAG, bool XBC, bool FORCE>
+template <class S, class R, bool ODD, bool DIAG, bool XBC, int FORM>
 static cudaError_t launch_phases_f(Lattice &L, const Args<S, R> &a) {
   cudaError_t e = launch_phi<S, R, ODD, XBC>(L, a);
   if (e != cudaSuccess) return e;
@@ -243,17 +244,20 @@ static cudaError_t launch_phases_f(Lattice &L, const Args<S, R> &a) {
   constexpr int NT = phase2_threads<R>();
   const int nwall = (L.nw + NT - 1) / NT, nedge = XBC ? (plane2 + NT - 1) / NT : 0;
   const long long grid = nwall + nedge + (L.N + NT - 1) / NT;
-  return launch_dependent(k_phase2<S, R, ODD, DIAG, XBC, FORCE>, (unsigned)grid, NT, 0, L.stream, a,
+  return launch_dependent(k_phase2<S, R, ODD, DIAG, XBC, FORM>, (unsigned)grid, NT, 0, L.stream, a,
                           nwall, nedge);
 }
 
 // The variant without body-force terms when F_ex = 0 (they vanish there).
 template <class S, class R, bool ODD, bool DIAG>
 static cudaError_t launch_phases(Lattice &L, const Args<S, R> &a) {
-  if (L.bc_on) return launch_phases_f<S, R, ODD, DIAG, true, true>(L, a);
+  if (L.bc_on) return launch_phases_f<S, R, ODD, DIAG, true, open_form<S>()>(L, a);
+  if constexpr (open_form<S>() == FORM_PLAIN) {
+    if (a.plain) return launch_phases_f<S, R, ODD, DIAG, false, FORM_PLAIN>(L, a);
+  }
   if (a.m.Fx == R(0) && a.m.Fy == R(0) && a.m.Fz == R(0))
-    return launch_phases_f<S, R, ODD, DIAG, false, false>(L, a);
-  return launch_phases_f<S, R, ODD, DIAG, false, true>(L, a);
+    return launch_phases_f<S, R, ODD, DIAG, false, FORM_NOFORCE>(L, a);
+  return launch_phases_f<S, R, ODD, DIAG, false, FORM_FORCE>(L, a);
 }
 
 template <class S, class R, bool ODD, bool DIAG>

@@ -10,10 +10,14 @@
 // the bulk cells of the same launch.  Where h stays in L2 between the two
 // kernels the second read costs no DRAM traffic.  Measured (GB300, us per
 // step, against the march, or the fused kernel where that could not run):
-// FP32 drop 32^3 6.2 (10.3), 64^3 14.4 (24.7), slit 1024 x 64 x 4 20.5 (31.7)
-// before dependent launches, channel 251 x 67 x 67 88 (153); BF16 sessile
-// 128^3 121 (139).  What bounds it: at 128^3 FP32 phase 1 takes 28.7 us, the
-// copy bandwidth; phase 2 117 us, 82 % of it; below 64^3 the launches.
+// FP32 drop 32^3 6.1 (10.3), sessile 64^3 14.6 (32.4), slit 1024 x 64 x 4 14.9
+// (31.7), constricted duct w = 48 29 (56), channel 251 x 67 x 67 75 (153), sessile
+// 128^3 136 (152); BF16 sessile 128^3 109 (138); FP64 sessile 64^3 303 (516).
+// What bounds it: at 128^3 FP32 phase 1 takes 28.7 us, the copy bandwidth, and
+// phase 2 runs at 82 to 90 % of it; at 16-bit storage the latency of the loads
+// (14 warps per SM) and 872 instructions per cell; at FP64 the FP64 rate; below
+// 64^3 the two launches and, in thin lattices, a wall node's chain of
+// instructions.
 //
 // A unit of work is one lane per cell: bulk cells by their linear index, wall
 // nodes by their record, boundary cells by their place in the two planes.
@@ -40,6 +44,19 @@ __host__ __device__ constexpr int phase2_threads() {
 template <class R>
 __host__ __device__ constexpr int phase2_blocks() {
   return sizeof(R) == 8 ? 8 : 7;
+}
+
+// Forms of the collision in phase 2: pair form without and with a body force
+// (packed at FP32, lean at FP64), and the per-direction form.
+enum { FORM_NOFORCE = 0, FORM_FORCE = 1, FORM_PLAIN = 2 };
+// FP32 lattices that the march's layout does not take (open x boundaries, nx
+// not a multiple of 4) have always had the per-direction form and keep it, so
+// that their results stay the same to the bit: through the switch of the
+// mobility correction (Eq. 4) one rounding can become 1e-3 of phi at an
+// interface cell within tens of steps.
+template <class S>
+__host__ __device__ constexpr int open_form() {
+  return std::is_same<S, float>::value ? FORM_PLAIN : FORM_FORCE;
 }
 
 // Diagnostic sums of one cell per lane over a warp, added to one of the copies
@@ -257,12 +274,14 @@ __device__ __forceinline__ void wall_update(const Args<S, R> &a, int rec, DiagAc
                                                         val, acc);
 }
 
-// (by every lane of the warp; on: the lane has a record)
-template <class S, class R, bool ODD, bool DIAG, bool XBC>
+// Phase 2 of a warp's wall nodes (every lane calls it; on: it has a record).
+template <class S, class R, bool ODD, bool DIAG, bool XBC, int FORM>
 __device__ __forceinline__ void phase2_wall(const Args<S, R> &a, int rec, bool on) {
   DiagAcc<R> acc;
   acc.zero();
-  if (on) wall_update<S, R, ODD, MODE_STEP, DIAG, XBC, COLL_X2>(a, rec, acc);
+  if (on)
+    wall_update<S, R, ODD, MODE_STEP, DIAG, XBC, FORM == FORM_PLAIN ? COLL_PLAIN : COLL_X2>(
+        a, rec, acc);
   if (DIAG) phase_diag<R>(diag_copy(a.diag), acc);
 }
 
@@ -283,16 +302,17 @@ __device__ __forceinline__ void phase2_edge(const Args<S, R> &a, int j) {
 // Phase 2 of bulk cell c (nothing for solid cells, wall nodes and boundary
 // cells, which have units of their own).  All loads are issued before the
 // flags decide, so that a warp waits for memory once (BF16 sessile 128^3:
-// 112.6 against 117.6 us per step).
-// Every lane of the warp calls it, those past the last cell too.
-template <class S, class R, bool ODD, bool DIAG, bool XBC, bool FORCE>
+// 112.6 against 117.6 us per step).  Every lane of the warp calls it, those
+// past the last cell too.
+template <class S, class R, bool ODD, bool DIAG, bool XBC, int FORM>
 __device__ __forceinline__ void phase2_bulk(const Args<S, R> &a, unsigned cell) {
-  // The diagnostics of FP32 cells are summed, by all lanes of the warp, before
-  // the collision needs the registers (sessile 128^3: 149 us per step, 157 when
-  // after it); at 16-bit storage, bound by instructions, the update is one
-  // branch and the sums come last (127 against 131 us; without diagnostics 109
-  // against 119).
-  constexpr bool MID = sizeof(S) > 2;
+  // FP32 without diagnostics keeps the lanes of a warp together between the
+  // fields and the update (sessile 128^3: 137 us per step against 142); at
+  // 16-bit storage one branch is faster (109 against 119).  With diagnostics
+  // the sums follow the update, as in finish_cell (127 us at BF16, 131 with
+  // them in between).
+  constexpr bool PLAIN = FORM == FORM_PLAIN;
+  constexpr bool MID = sizeof(S) > 2 && !DIAG && !PLAIN;
   bool on = cell < (unsigned)a.N;
   if (!MID && !DIAG && !on) return;
   const int c = on ? (int)cell : 0;
@@ -322,9 +342,9 @@ __device__ __forceinline__ void phase2_bulk(const Args<S, R> &a, unsigned cell) 
   };
   auto update = [&] {
     if constexpr (std::is_same<R, float>::value)
-      collide_pairs_x2<FORCE>(m, h, g, mc, val[0], gx, gy, gz, lap);
+      collide_pairs_x2<FORM == FORM_FORCE>(m, h, g, mc, val[0], gx, gy, gz, lap);
     else
-      collide_pairs_lean<R, FORCE>(m, h, g, mc, val[0], gx, gy, gz, lap);
+      collide_pairs_lean<R, FORM == FORM_FORCE>(m, h, g, mc, val[0], gx, gy, gz, lap);
     store_cell<S, R, ODD>(a, c, 0u, 0, nb, h, g, val, false);
   };
   DiagAcc<R> acc;
@@ -332,14 +352,17 @@ __device__ __forceinline__ void phase2_bulk(const Args<S, R> &a, unsigned cell) 
   auto sums = [&] { diag_cell<S, R>(a, x, y, z, false, 0u, val[0], val[1], mc, acc); };
   if constexpr (MID) {
     if (on) on = load();
-    if (on) {
-      fields();
-      if (DIAG) sums();
-    }
-    if (DIAG) phase_diag<R>(diag_copy(a.diag), acc);
+    if (on) fields();
     if (on) update();
   } else {
-    if (on && load()) {
+    if constexpr (PLAIN) {
+      // finish_cell with the flags as read, not as known to have no F_WALL:
+      // the sums that its wall corrections add to then stay uncontracted, as
+      // in every build of this form (see open_form)
+      if (on && load())
+        finish_cell<S, R, ODD, MODE_STEP, DIAG, XBC, COLL_PLAIN>(a, x, y, z, c, a.flags[c], 0u, 0,
+                                                                 nb, h, g, val[0], val, acc);
+    } else if (on && load()) {
       fields();
       if (DIAG) sums();
       update();
@@ -373,7 +396,7 @@ __global__ void __launch_bounds__(PH_NT1)
 // the first: phase 1 read the last ones' h most recently, and the next phase
 // 1 begins with the h written last (144^3 FP32: 201 instead of 210 us, BF16
 // 166 instead of 172).
-template <class S, class R, bool ODD, bool DIAG, bool XBC, bool FORCE>
+template <class S, class R, bool ODD, bool DIAG, bool XBC, int FORM>
 __global__ void __launch_bounds__(phase2_threads<R>(), phase2_blocks<R>())
     k_phase2(const __grid_constant__ Args<S, R> a, int nwall, int nedge) {
   constexpr int NT = phase2_threads<R>();
@@ -382,12 +405,12 @@ __global__ void __launch_bounds__(phase2_threads<R>(), phase2_blocks<R>())
   const int u = blockIdx.x;
   if (u < nwall) {
     const int rec = u * NT + threadIdx.x;
-    phase2_wall<S, R, ODD, DIAG, XBC>(a, rec, rec < a.nw);
+    phase2_wall<S, R, ODD, DIAG, XBC, FORM>(a, rec, rec < a.nw);
   } else if (XBC && u < nwall + nedge) {
     const int j = (u - nwall) * NT + threadIdx.x;
     if (j < 2 * a.ny * a.nz) phase2_edge<S, R, ODD>(a, j);
   } else {
-    phase2_bulk<S, R, ODD, DIAG, XBC, FORCE>(a, (gridDim.x - 1 - u) * NT + threadIdx.x);
+    phase2_bulk<S, R, ODD, DIAG, XBC, FORM>(a, (gridDim.x - 1 - u) * NT + threadIdx.x);
   }
 }
 
@@ -501,16 +524,16 @@ __global__ void __launch_bounds__(PH_NT1)
   }
 }
 
-template <class S, class R, bool ODD, bool DIAG, bool XBC>
+template <class S, class R, bool ODD, bool DIAG, bool XBC, int FORM>
 __device__ __forceinline__ void batch_update(const Args<S, R> &a, const int4 &it) {
   for (int j0 = it.z; j0 < it.z + it.w; j0 += phase2_threads<R>()) {
     const int j = j0 + (int)threadIdx.x;
     // (an item of bulk cells ends at the lattice's last cell or at a multiple
     // of the block)
     if (it.y == UPD_BULK)
-      phase2_bulk<S, R, ODD, DIAG, XBC, true>(a, j);
+      phase2_bulk<S, R, ODD, DIAG, XBC, FORM>(a, j);
     else if (it.y == UPD_WALL)
-      phase2_wall<S, R, ODD, DIAG, XBC>(a, j, j < it.z + it.w);
+      phase2_wall<S, R, ODD, DIAG, XBC, FORM>(a, j, j < it.z + it.w);
     else if (XBC && j < it.z + it.w)
       phase2_edge<S, R, ODD>(a, j);
   }
@@ -528,10 +551,18 @@ __global__ void __launch_bounds__(phase2_threads<R>(), phase2_blocks<R>())
   if (blockIdx.x == 0 && threadIdx.x == 0) *bstep += 1;
   // the first item of a lattice's bulk cells zeroes its next accumulator
   if (DIAG && it.y == UPD_BULK && it.z == 0) zero_diag(a.diag_zero);
+  constexpr int FORM = XBC ? open_form<S>() : FORM_FORCE;
+  if (!XBC && open_form<S>() == FORM_PLAIN && a.plain) {
+    if (p)
+      batch_update<S, R, true, DIAG, XBC, open_form<S>()>(a, it);
+    else
+      batch_update<S, R, false, DIAG, XBC, open_form<S>()>(a, it);
+    return;
+  }
   if (p)
-    batch_update<S, R, true, DIAG, XBC>(a, it);
+    batch_update<S, R, true, DIAG, XBC, FORM>(a, it);
   else
-    batch_update<S, R, false, DIAG, XBC>(a, it);
+    batch_update<S, R, false, DIAG, XBC, FORM>(a, it);
 }
 
 // Sum of the copies of an accumulator and the device error flag, as the record
