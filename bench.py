@@ -335,7 +335,7 @@ def main_channels(args):
         cells += g.N
     ev = lambda: torch.cuda.Event(enable_timing=True)  # noqa: E731
 
-    # per-lattice loop: one fused launch per lattice per step
+    # per-lattice loop: each lattice stepped by itself
     for L in lats:
         L.step(args.warmup)
     a, b = ev(), ev()
@@ -423,9 +423,9 @@ def serve_trace(server, prepared, trace):
 
 def main_serve(args):
     """Critical-pressure solves served from a Poisson trace: continuous
-    batching (one persistent batch kernel per step over all resident
+    batching (one batch call per tick over all resident
     requests, admission by HBM budget) against the plain server (one request
-    at a time, FP32, one fused launch per step) on the same trace."""
+    at a time, FP32) on the same trace."""
     import torch
     from paper_2512_01032_gb300 import pflb, shard
     world, rank = init_ranks()

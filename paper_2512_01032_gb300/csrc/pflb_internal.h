@@ -76,7 +76,6 @@ struct Lattice {
   int64_t dev_bytes = 0;
 };
 
-// Device side of a batch of lattices stepped by one persistent kernel.
 // Open x boundaries of one lattice as the boundary-state kernels take them.
 struct XbcSpec {
   int type[2];        // 1 pressure (P given), 2 velocity (u and phi given); 0 closed

@@ -2,8 +2,8 @@
 // and batch C API (host code only).
 //
 // Each tick: set each resident request's ramp force for its own step count
-// and launch steps_per_tick steps for all of them (one persistent batch
-// kernel per step, or one fused launch per request); while the GPU runs,
+// and launch steps_per_tick steps for all of them (one batch call,
+// or one step call per request); while the GPU runs,
 // admit queued requests in arrival order while the budget holds; then
 // synchronise once, read each stepped request's diagnostics of the last
 // step and retire the finished ones.  The batch is rebuilt only when the

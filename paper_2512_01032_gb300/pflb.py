@@ -464,7 +464,7 @@ class Lattice:
 
 
 class Batch:
-    """Many lattices advanced together by one persistent kernel (the lattices
+    """Many lattices advanced together (the lattices
     stay owned by the caller and must outlive the batch)."""
 
     def __init__(self, lattices, stream=None):
