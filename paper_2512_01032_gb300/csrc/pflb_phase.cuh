@@ -51,7 +51,8 @@ __host__ __device__ constexpr int phase2_blocks() {
 enum { FORM_NOFORCE = 0, FORM_FORCE = 1, FORM_PLAIN = 2 };
 // FP32 lattices that the march's layout does not take (open x boundaries, nx
 // not a multiple of 4) have always had the per-direction form and keep it, so
-// that their results stay the same to the bit: through the switch of the
+// that their results stay the same to the bit (a step with diagnostics, where
+// the compiler contracts differently, to its rounding): through the switch of the
 // mobility correction (Eq. 4) one rounding can become 1e-3 of phi at an
 // interface cell within tens of steps.  Packed pairs / per direction: channel
 // 251 x 67 x 67 76 / 91 us per step, 25 steps of an open duct 192 x 50 x 50
