@@ -582,7 +582,7 @@ __device__ __forceinline__ R cell_phi(const Args<S, R> &a, int c) {
     if (f & F_BC) return a.bcm[bc_index(a, c % a.nx, c / a.nx)];  // phi_b
   }
   R h[Q];
-  ld_h_cell<S, R>(a.hin, c, h);
+  ld_h_cell_ro<S, R>(a.hin, c, h);
   R s = R(0);
 #pragma unroll
   for (int i = 0; i < Q; ++i) s += h[i];
@@ -635,7 +635,7 @@ __global__ void __launch_bounds__(256) k_cell(const __grid_constant__ Args<S, R>
       nb.init(x, y, z, a.nx, a.ny, a.nz);
       R h[Q], val[Q];
       R phi = R(0);
-      ld_h_cell<S, R>(a.hin, c, h);
+      ld_h_cell_ro<S, R>(a.hin, c, h);
 #pragma unroll
       for (int i = 0; i < Q; ++i) phi += h[i];
 #pragma unroll
@@ -698,7 +698,7 @@ __device__ __forceinline__ void march_tile(const Args<S, R> &a, int x0, int y0, 
       const uint8_t f = a.flags[c];
       if (!(f & F_SOLID)) {
         R h[Q], val[Q];
-        ld_h_cell<S, R>(a.hin, c, h);
+        ld_h_cell_ro<S, R>(a.hin, c, h);
         const R *p0 = sphi + (((z % 3) + 3) % 3) * PS;
         const R *pm = sphi + ((((z - 1) % 3) + 3) % 3) * PS;
         const R *pp = sphi + ((((z + 1) % 3) + 3) % 3) * PS;

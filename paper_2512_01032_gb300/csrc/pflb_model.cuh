@@ -114,9 +114,12 @@ template <> struct Store<float> {
   static __device__ __forceinline__ float ld(const float *p) { return *p; }
   static __device__ __forceinline__ void st(float *p, float v) { *p = v; }
 };
-// Loads of data that no thread writes during the launch (the h buffer being
-// read): may go through the read-only data path.  In-place arrays (g) must
-// not, since the compiler may then move such loads past aliasing stores.
+// Loads of data that nothing writes while the kernel exists (the h buffer
+// being read, in a kernel that starts after the one before it has ended): may
+// go through the read-only data path.  In-place arrays (g) must not, since the
+// compiler may then move such loads past aliasing stores; nor may anything in
+// a dependent launch (launch_ready), whose blocks exist while the kernel
+// before still writes.
 template <class S> __device__ __forceinline__ S ld_ro(const S *p) { return __ldg(p); }
 
 // ------------------------------------------------------------ codecs
@@ -209,10 +212,17 @@ template <class S, class R> __device__ __forceinline__ R ld_g(const S *p, int i)
 template <class S, class R> __device__ __forceinline__ void st_g(S *p, int i, R v) {
   *p = enc_pop<S, R>(v, i);
 }
-// Loads all 19 h of cell c from direction bases hb (read-only path); the
-// rest population of the 16-bit formats is high part + remainder.
+// Loads all 19 h of cell c from direction bases hb; the rest population of
+// the 16-bit formats is high part + remainder.
 template <class S, class R>
 __device__ __forceinline__ void ld_h_cell(const S *const *hb, int c, R h[Q]) {
+#pragma unroll
+  for (int i = 0; i < Q; ++i) h[i] = dec_pop<S, R>(hb[i][c], i);
+  if constexpr (Codec<S>::narrow) h[0] += dec_pop<S, R>(hb[Q][c], 0);
+}
+// The same by the read-only path (see ld_ro for who may).
+template <class S, class R>
+__device__ __forceinline__ void ld_h_cell_ro(const S *const *hb, int c, R h[Q]) {
 #pragma unroll
   for (int i = 0; i < Q; ++i) h[i] = dec_pop<S, R>(ld_ro<S>(hb[i] + c), i);
   if constexpr (Codec<S>::narrow) h[0] += dec_pop<S, R>(ld_ro<S>(hb[Q] + c), 0);

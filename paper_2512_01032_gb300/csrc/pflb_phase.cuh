@@ -130,7 +130,12 @@ __device__ __forceinline__ void phase_diag(double *diag, const DiagAcc<R> &d) {
 }
 
 // Dependent launches: a block lets the next kernel of the stream be set up
-// at once, and itself waits here until the one before has finished.
+// at once, and itself waits here until the one before has finished.  So a
+// block exists while the kernel before still writes phi, h, g or the
+// diagnostic copies, and the read-only path (the read-only load intrinsic,
+// ld_ro, restrict pointers to const) is only for memory that stays the same
+// for as long as the kernel exists: every kernel that waits here, and every
+// function that it calls, uses ordinary loads, which stay behind the wait.
 __device__ __forceinline__ void launch_ready() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -168,7 +173,7 @@ __device__ __forceinline__ void phi_cells(const Args<S, R> &a, const XbcSpec &sp
     uint4 q[h_slots<S>()];
 #pragma unroll
     for (int i = 0; i < h_slots<S>(); ++i)
-      q[i] = __ldg(reinterpret_cast<const uint4 *>(a.hin[i] + c));
+      q[i] = *reinterpret_cast<const uint4 *>(a.hin[i] + c);
     if constexpr (V == 8) {
       const uint2 w = *reinterpret_cast<const uint2 *>(a.flags + c);
       memcpy(f, &w, 8);
@@ -329,9 +334,9 @@ __device__ __forceinline__ void phase2_bulk(const Args<S, R> &a, unsigned cell) 
   Macro<R> mc;
   auto load = [&] {
     const uint8_t f = a.flags[c];
-    val[0] = __ldg(a.phi + c);
+    val[0] = a.phi[c];
 #pragma unroll
-    for (int i = 1; i < Q; ++i) val[i] = __ldg(a.phi + (c + nb.off(i)));
+    for (int i = 1; i < Q; ++i) val[i] = a.phi[c + nb.off(i)];
     gather_g<S, R, ODD>(a, c, 0u, 0, nb, g);
     ld_h_cell<S, R>(a.hin, c, h);
     return !(f & (F_SOLID | F_WALL | (XBC ? F_BC : 0)));
@@ -476,9 +481,9 @@ __global__ void __launch_bounds__(phase2_threads<R>())
     Nbr nb;
     nb.init(x, y, z, a.nx, a.ny, a.nz);
     R g[Q], val[Q], gx, gy, gz, lap;
-    val[0] = __ldg(a.phi + c);
+    val[0] = a.phi[c];
 #pragma unroll
-    for (int i = 1; i < Q; ++i) val[i] = __ldg(a.phi + (c + nb.off(i)));
+    for (int i = 1; i < Q; ++i) val[i] = a.phi[c + nb.off(i)];
     gather_g<S, R, ODD>(a, c, 0u, 0, nb, g);
     cd_stencil(val, gx, gy, gz, lap);
     const Macro<R> mc = macros(a.m, g, val[0], gx, gy, gz, lap);
@@ -507,9 +512,8 @@ __device__ __forceinline__ const Args<S, R> &batch_args(unsigned char *smem,
 // (boundary ramps), advanced by phase 2.
 template <class S, class R, bool XBC>
 __global__ void __launch_bounds__(PH_NT1)
-    k_batch_phase1(const Args<S, R> *__restrict__ descs, const int *__restrict__ par0,
-                   const int4 *__restrict__ items, const XbcSpec *__restrict__ specs,
-                   const int *bstep, int tpar) {
+    k_batch_phase1(const Args<S, R> *descs, const int *par0, const int4 *items,
+                   const XbcSpec *specs, const int *bstep, int tpar) {
   __shared__ __align__(16) unsigned char smem[sizeof(Args<S, R>)];
   launch_ready();
   const int4 it = items[blockIdx.x];
@@ -546,8 +550,8 @@ __device__ __forceinline__ void batch_update(const Args<S, R> &a, const int4 &it
 
 template <class S, class R, bool DIAG, bool XBC>
 __global__ void __launch_bounds__(phase2_threads<R>(), phase2_blocks<R>())
-    k_batch_phase2(const Args<S, R> *__restrict__ descs, const int *__restrict__ par0,
-                   const int4 *__restrict__ items, int *bstep, int tpar) {
+    k_batch_phase2(const Args<S, R> *descs, const int *par0, const int4 *items, int *bstep,
+                   int tpar) {
   __shared__ __align__(16) unsigned char smem[sizeof(Args<S, R>)];
   launch_ready();
   const int4 it = items[blockIdx.x];
@@ -573,7 +577,7 @@ __global__ void __launch_bounds__(phase2_threads<R>(), phase2_blocks<R>())
 // Sum of the copies of an accumulator and the device error flag, as the record
 // that a diagnostics read returns (256 threads).  out may be page-locked host
 // memory: a synchronous read is then this kernel and a wait, without copies.
-static __global__ void k_diag_fold(const double *__restrict__ copies, const int *err, int64_t step,
+static __global__ void k_diag_fold(const double *copies, const int *err, int64_t step,
                                    pflb_diag_raw_t *out) {
   __shared__ double part[8][32];
   launch_ready();

@@ -149,7 +149,7 @@ __device__ __forceinline__ void wall_node(const Args<S, R> &a, int rec, DiagAcc<
   Nbr nb;
   nb.init(x, y, z, a.nx, a.ny, a.nz);
   R h[Q], val[Q];
-  ld_h_cell<S, R>(a.hin, c, h);
+  ld_h_cell_ro<S, R>(a.hin, c, h);
   R phi = R(0);
 #pragma unroll
   for (int i = 0; i < Q; ++i) phi += h[i];
