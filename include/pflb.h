@@ -74,8 +74,9 @@ enum { PFLB_FIELD_PHI = 0, PFLB_FIELD_RHO = 1, PFLB_FIELD_P = 2,
  *     one fused z-marching kernel instead, each thread's populations of the
  *     next planes copied into shared memory one plane ahead (cp.async in
  *     16-byte chunks).  Both use the pair form of the collision, but for
- *     FP32 lattices with open x boundaries or nx not a multiple of 4, which
- *     take it per direction as PFLB_KERNEL_FUSED does;
+ *     FP32, FP16 and BF16 lattices with open x boundaries or nx not a
+ *     multiple of 4, which take it per direction, to the bit as
+ *     PFLB_KERNEL_FUSED does;
  *   PFLB_KERNEL_FUSED: one fused z-marching pass with direct loads;
  *   PFLB_KERNEL_TWOPASS: a phi pass followed by a per-cell pass;
  *   PFLB_KERNEL_FUSED_TMA: the fused pass with h staged through shared

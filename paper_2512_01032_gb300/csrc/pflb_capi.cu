@@ -1372,10 +1372,12 @@ static pflb_status batch_run(pflb_batch *b, int64_t nsteps, bool diag_last) {
     Lattice *L = b->lats[l];
     const cudaStream_t own = L->stream;
     L->stream = b->dev.stream;
+    L->in_batch = true;
     cudaError_t e = cudaSuccess;
     for (int64_t t = 0; t < nsteps && e == cudaSuccess; ++t)
       e = do_step(L, diag_last && t == nsteps - 1);
     L->stream = own;
+    L->in_batch = false;
     BCK(b, e);
   }
   // later work on each lattice's own stream comes after the batch

@@ -56,6 +56,7 @@ struct Lattice {
   int diag_every = 0;         // pflb_step accumulates diagnostics every k-th step
   int kernel = PFLB_KERNEL_PIPE;
   bool march = false;         // the default kind marches where it can (pipe_kernel_runs)
+  bool in_batch = false;      // while a batch steps it
   int bx = 32, by = 4, lz = 16;   // lz: planes per block in effect
   int lz_req = 0;                  // requested planes per block, 0 = automatic
   // open x boundaries (reading R22)

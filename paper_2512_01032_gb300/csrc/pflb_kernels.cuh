@@ -27,8 +27,9 @@ namespace pflb {
 enum { MODE_STEP = 0, MODE_MACRO = 1 };
 // Collision forms: per direction (collide), per opposite pair
 // (collide_pairs), pairs in packed FP32 lanes with and without the body
-// force terms (collide_pairs_x2; FP32 arithmetic only, else collide_pairs).
-enum { COLL_PLAIN = 0, COLL_PAIRS = 1, COLL_X2 = 2, COLL_X2_NOF = 3 };
+// force terms (collide_pairs_x2; FP32 arithmetic only, else collide_pairs);
+// per direction with fixed roundings (collide's RN, FP32 arithmetic only).
+enum { COLL_FIXED = -1, COLL_PLAIN = 0, COLL_PAIRS = 1, COLL_X2 = 2, COLL_X2_NOF = 3 };
 
 // Blocks of 256 threads per SM the batch kernel is compiled for (sets its
 // register cap: 128).
@@ -66,6 +67,7 @@ struct Args {
   int nw;
   FastDiv dx, dxy;       // by nx and by nx ny
   int plain;             // nx not a multiple of 4 (open_form)
+  int batch;             // stepped in a batch (collide's RN)
   const S *hin[Q + 1];   // direction bases of the h buffer being read (+ rest remainder)
   S *hout[Q + 1];        // direction bases of the h buffer being written
   S *g[Q];           // direction bases of the g buffer (in place)
@@ -250,12 +252,13 @@ __device__ __forceinline__ void diag_cell(const Args<S, R> &a, int x, int y, int
 // once its populations are gathered: h[] and g[] hold the streamed
 // populations, phi = sum h, val[1..18] the phi of the 18 neighbours
 // (anything for solid ones; with HAVE, their ghosts), lm/rec the wall data (0
-// for bulk cells).
+// for bulk cells), hraw the h as stored (COLL_FIXED at FP16 storage).
 template <class S, class R, bool ODD, int MODE, bool DIAG, bool XBC = false, int PAIRS = COLL_PLAIN,
           bool HAVE = false>
 __device__ __forceinline__ void finish_cell(const Args<S, R> &a, int x, int y, int z, int c,
                                             uint8_t f, uint32_t lm, int rec, const Nbr &nb,
-                                            R h[Q], R g[Q], R phi, R val[Q], DiagAcc<R> &acc) {
+                                            R h[Q], R g[Q], R phi, R val[Q], DiagAcc<R> &acc,
+                                            const R *hraw = nullptr) {
   const Model<R> &m = a.m;
   if constexpr (XBC) {
     if (f & F_BC) {
@@ -356,6 +359,9 @@ __device__ __forceinline__ void finish_cell(const Args<S, R> &a, int x, int y, i
     collide_pairs_x2<PAIRS == COLL_X2>(m, h, g, mc, phi, gx, gy, gz, lap);
   else if constexpr (PAIRS >= COLL_PAIRS)
     collide_pairs(m, h, g, mc, phi, gx, gy, gz, lap);
+  else if constexpr (PAIRS == COLL_FIXED)
+    collide<R, DIAG ? RN_DIAG : RN_STEP>(m, h, g, mc, phi, gx, gy, gz, lap, hraw,
+                                             a.batch);
   else
     collide(m, h, g, mc, phi, gx, gy, gz, lap);
   store_cell<S, R, ODD>(a, c, lm, rec, nb, h, g, val,

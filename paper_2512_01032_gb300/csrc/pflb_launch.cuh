@@ -56,6 +56,7 @@ static Args<S, R> make_args(const Lattice &L, int parity) {
   a.dx = fast_div((uint32_t)L.nx);
   a.dxy = fast_div((uint32_t)L.nx * (uint32_t)L.ny);
   a.plain = L.nx % 4 != 0;
+  a.batch = L.in_batch;
   const int rd = parity;
   for (int i = 0; i < Q + 1; ++i) {
     const bool have = i < h_slots<S>();
@@ -441,6 +442,7 @@ void batch_build_descs(Lattice *const *lats, int n, char *host) {
   for (int l = 0; l < n; ++l) {
     for (int p = 0; p < 2; ++p) {
       Args<S, R> a = make_args<S, R>(*lats[l], p);
+      a.batch = 1;
       a.diag = diag_acc(*lats[l], (int)(lats[l]->ndiag & 1));
       a.diag_zero = diag_acc(*lats[l], (int)((lats[l]->ndiag + 1) & 1));
       std::memcpy(host + (2 * (size_t)l + p) * sizeof(Args<S, R>), &a, sizeof a);

@@ -174,6 +174,15 @@ __device__ __forceinline__ R dec_pop(S v, int i) {
   else
     return Codec<S>::template to<R>(v);
 }
+// The same with the weight's product rounded by itself, whatever it is added
+// to (the compiler may otherwise contract the two).
+template <class S, class R>
+__device__ __forceinline__ R dec_pop_rn(S v, int i) {
+  if constexpr (Codec<S>::scaled)
+    return __fmul_rn(Codec<S>::template to<R>(v), R(w_of(i)));
+  else
+    return Codec<S>::template to<R>(v);
+}
 template <class S, class R>
 __device__ __forceinline__ S enc_pop(R v, int i) {
   if constexpr (Codec<S>::scaled)
@@ -359,13 +368,17 @@ __device__ __forceinline__ R tau_mix(const Model<R> &m, R phi) {
   return (R(1) - F) * m.tau_L + F * m.tau_H;
 }
 
-// Local mobility correction (Eq. 4).
+// Local mobility correction (Eq. 4): its windows, and the whole.
 template <class R>
-__device__ __forceinline__ R delta_theta(const Model<R> &m, R phi, R gnorm, R lap) {
+__device__ __forceinline__ R delta_windows(const Model<R> &m, R phi, R lap) {
   R Y1 = fminf_(clamp01_((phi - m.phi_M) * m.inv_D), clamp01_((R(1) - phi) * m.inv_D));
   R Y2 = fminf_(clamp01_(phi * m.inv_D), clamp01_((m.phi_m - phi) * m.inv_D));
   R s = div_(lap, abs_(lap) + m.eps);  // reading R4: the sign of lap, regularised
-  return m.gamma * m.theta_coef * gnorm * ((R(1) + s) * Y1 + (R(1) - s) * Y2);
+  return (R(1) + s) * Y1 + (R(1) - s) * Y2;
+}
+template <class R>
+__device__ __forceinline__ R delta_theta(const Model<R> &m, R phi, R gnorm, R lap) {
+  return m.gamma * m.theta_coef * gnorm * delta_windows(m, phi, lap);
 }
 
 // Both collisions of one cell, in place on h[] and g[] (Eqs. 1-11):
@@ -378,16 +391,32 @@ __device__ __forceinline__ R delta_theta(const Model<R> &m, R phi, R gnorm, R la
 //      Pi = sum c c (g - E + K/2).  Gamma_i - w_i is evaluated directly so
 //      that the heavy phase (rho = 1) does not cancel the pressure part.
 // Gamma_i is shared by the two sets.
-template <class R>
+// RN other than RN_FREE writes the roundings of the h set out, FP32 arithmetic
+// only: which of two products is contracted into their sum is otherwise the
+// compiler's choice, another one in every kernel.  They are the choices that it
+// made in k_fused, which stepped such lattices first, for steps without and
+// with diagnostics, and in the tile march that stepped them in batches (batch).
+// At FP16 those kernels also contracted the decoding of directions 13 to 17 (14
+// to 17 in plain batch steps) into their update; hraw holds them as stored.
+enum { RN_FREE = 0, RN_STEP = 1, RN_DIAG = 2 };
+template <class R, int RN = RN_FREE>
 __device__ __forceinline__ void collide(const Model<R> &m, R h[Q], R g[Q], const Macro<R> &mc,
-                                        R phi, R gx, R gy, R gz, R lap) {
+                                        R phi, R gx, R gy, R gz, R lap,
+                                        const R *hraw = nullptr, int batch = 0) {
   const R ux = mc.ux, uy = mc.uy, uz = mc.uz;
   // interface normal and theta (Eqs. 2-4)
   const R gn2 = gx * gx + gy * gy + gz * gz;
   const R gnorm = sqrt_(gn2);
   const R inv = div_(R(1), gnorm + m.eps);
-  R th = m.theta_coef * (R(1) - R(4) * (phi - R(0.5)) * (phi - R(0.5)));
-  if (m.mobility_corr) th += delta_theta(m, phi, gnorm, lap);
+  const R win = R(1) - R(4) * (phi - R(0.5)) * (phi - R(0.5));
+  R th = m.theta_coef * win;
+  if constexpr (RN == RN_FREE) {
+    if (m.mobility_corr) th += delta_theta(m, phi, gnorm, lap);
+  } else if (m.mobility_corr) {
+    const R cf = m.gamma * m.theta_coef * gnorm, dw = delta_windows(m, phi, lap);
+    th = RN == RN_STEP || batch ? __fmaf_rn(cf, dw, __fmul_rn(m.theta_coef, win))
+                                : __fmaf_rn(m.theta_coef, win, __fmul_rn(cf, dw));
+  }
   const R thn = th * inv;  // theta * n = thn * grad
   const R om = m.inv_tau_phi;
   const R uu15 = R(1.5) * (ux * ux + uy * uy + uz * uz);
@@ -407,8 +436,15 @@ __device__ __forceinline__ void collide(const Model<R> &m, R h[Q], R g[Q], const
     // h
     if (i != 0) {
       const R cgr = R(c0) * gx + R(c1) * gy + R(c2) * gz;  // c . grad phi
-      const R heq = phi * G + (thn * wi) * cgr;
-      h[i] = h[i] + om * (heq - h[i]);
+      if constexpr (RN == RN_FREE) {
+        const R heq = phi * G + (thn * wi) * cgr;
+        h[i] = h[i] + om * (heq - h[i]);
+      } else {
+        const R heq = __fmaf_rn(__fmul_rn(thn, wi), cgr, __fmul_rn(phi, G));
+        h[i] = hraw && i <= 17 && (i >= 14 || (i == 13 && (RN == RN_DIAG || !batch)))
+                   ? __fmaf_rn(hraw[i], wi, __fmul_rn(om, __fmaf_rn(-hraw[i], wi, heq)))
+                   : __fmaf_rn(om, __fsub_rn(heq, h[i]), h[i]);
+      }
       rest -= h[i];
     }
     // g

@@ -49,17 +49,38 @@ __host__ __device__ constexpr int phase2_blocks() {
 // Forms of the collision in phase 2: pair form without and with a body force
 // (packed at FP32, lean at FP64), and the per-direction form.
 enum { FORM_NOFORCE = 0, FORM_FORCE = 1, FORM_PLAIN = 2 };
-// FP32 lattices that the march's layout does not take (open x boundaries, nx
-// not a multiple of 4) have always had the per-direction form and keep it, so
-// that their results stay the same to the bit (a step with diagnostics, where
-// the compiler contracts differently, to its rounding): through the switch of the
-// mobility correction (Eq. 4) one rounding can become 1e-3 of phi at an
-// interface cell within tens of steps.  Packed pairs / per direction: channel
-// 251 x 67 x 67 76 / 91 us per step, 25 steps of an open duct 192 x 50 x 50
-// 1.08 / 1.32 ms.
+// Lattices in FP32 arithmetic that the march's layout does not take (open x
+// boundaries, nx not a multiple of 4) have always had the per-direction form
+// and keep it, with k_fused's roundings (COLL_FIXED), so that their results
+// stay the same to the bit: through the switch of the mobility correction
+// (Eq. 4) one rounding can become 1e-3 of phi at an interface cell within tens
+// of steps.  Packed pairs / per direction, us per step: FP32 channel 251 x 67 x
+// 67 76 / 87, open duct 192 x 50 x 50 39 / 44; BF16 66 / 72 and 34.5 / 38.3,
+// sessile 98^3 48.6 / 59.1; FP16 72 / 84, 36 / 42, 52 / 68.
 template <class S>
 __host__ __device__ constexpr int open_form() {
-  return std::is_same<S, float>::value ? FORM_PLAIN : FORM_FORCE;
+  return sizeof(S) <= 4 ? FORM_PLAIN : FORM_FORCE;
+}
+
+// The h of a cell as stored, where COLL_FIXED needs them (FP16, the only
+// storage whose decoding rounds).
+template <class S, class R>
+__device__ __forceinline__ const R *raw_h(const Args<S, R> &a, int c, R raw[Q]) {
+  if constexpr (Codec<S>::scaled) {
+#pragma unroll
+    for (int i = 13; i <= 17; ++i) raw[i] = Codec<S>::template to<R>(a.hin[i][c]);
+    return raw;
+  }
+  return nullptr;
+}
+
+// g of bulk cell c (A-A), for the packed forms: every weight's product rounded
+// by itself, as when the march read them from shared memory.
+template <class S, class R, bool ODD>
+__device__ __forceinline__ void gather_bulk(const Args<S, R> &a, int c, const Nbr &nb, R g[Q]) {
+#pragma unroll
+  for (int k = 0; k < Q; ++k)
+    g[k] = dec_pop_rn<S, R>(ODD ? a.g[opp_of(k)][c + nb.off(opp_of(k))] : a.g[k][c], k);
 }
 
 // Diagnostic sums of one cell per lane over a warp, added to one of the copies
@@ -275,11 +296,17 @@ __device__ __forceinline__ void wall_update(const Args<S, R> &a, int rec, DiagAc
     if (k != 0 && ((lm >> opp_of(k)) & 1u)) p = a.wp_rd + ((k - 1) * nw + rec);
     g[k] = ld_g<S, R>(p, k);
   }
-  R phi = R(0);
+  R phi = R(0), raw[Q];
+  const R *hraw = nullptr;
+  if constexpr (PAIRS == COLL_FIXED) {
+    phi = a.phi[c];  // (as k_fused: the sum that the neighbours see)
+    hraw = raw_h<S, R>(a, c, raw);
+  } else {
 #pragma unroll
-  for (int i = 0; i < Q; ++i) phi += h[i];
+    for (int i = 0; i < Q; ++i) phi += h[i];
+  }
   finish_cell<S, R, ODD, MODE, DIAG, false, PAIRS, true>(a, x, y, z, c, f, lm, rec, nb, h, g, phi,
-                                                        val, acc);
+                                                        val, acc, hraw);
 }
 
 // Phase 2 of a warp's wall nodes (every lane calls it; on: it has a record).
@@ -288,7 +315,7 @@ __device__ __forceinline__ void phase2_wall(const Args<S, R> &a, int rec, bool o
   DiagAcc<R> acc;
   acc.zero();
   if (on)
-    wall_update<S, R, ODD, MODE_STEP, DIAG, XBC, FORM == FORM_PLAIN ? COLL_PLAIN : COLL_X2>(
+    wall_update<S, R, ODD, MODE_STEP, DIAG, XBC, FORM == FORM_PLAIN ? COLL_FIXED : COLL_X2>(
         a, rec, acc);
   if (DIAG) phase_diag<R>(diag_copy(a.diag), acc);
 }
@@ -337,7 +364,10 @@ __device__ __forceinline__ void phase2_bulk(const Args<S, R> &a, unsigned cell) 
     val[0] = a.phi[c];
 #pragma unroll
     for (int i = 1; i < Q; ++i) val[i] = a.phi[c + nb.off(i)];
-    gather_g<S, R, ODD>(a, c, 0u, 0, nb, g);
+    if constexpr (PLAIN)
+      gather_g<S, R, ODD>(a, c, 0u, 0, nb, g);
+    else
+      gather_bulk<S, R, ODD>(a, c, nb, g);
     ld_h_cell<S, R>(a.hin, c, h);
     return !(f & (F_SOLID | F_WALL | (XBC ? F_BC : 0)));
   };
@@ -369,9 +399,11 @@ __device__ __forceinline__ void phase2_bulk(const Args<S, R> &a, unsigned cell) 
       // finish_cell with the flags as read, not as known to have no F_WALL:
       // the sums that its wall corrections add to then stay uncontracted, as
       // in every build of this form (see open_form)
-      if (on && load())
-        finish_cell<S, R, ODD, MODE_STEP, DIAG, XBC, COLL_PLAIN>(a, x, y, z, c, a.flags[c], 0u, 0,
-                                                                 nb, h, g, val[0], val, acc);
+      if (on && load()) {
+        R raw[Q];
+        finish_cell<S, R, ODD, MODE_STEP, DIAG, XBC, COLL_FIXED>(
+            a, x, y, z, c, a.flags[c], 0u, 0, nb, h, g, val[0], val, acc, raw_h<S, R>(a, c, raw));
+      }
     } else if (on && load()) {
       fields();
       if (DIAG) sums();
