@@ -393,7 +393,7 @@ pflb_status pflb_batch_create(pflb_lattice *const *lattices, int count, void *cu
                               pflb_batch **out);
 
 /* Launch shape of the groups: a work item of bulk cells holds bx * by * lz / 16
- * of them (bx and by under the rules of pflb_set_kernel); zeros keep the
+ * of them, a quarter of that at FP64 (bx and by under the rules of pflb_set_kernel); zeros keep the
  * current values (default 32 x 4 x 16).  blocks_per_sm is accepted (>= 0) and
  * bounds the value that pflb_batch_tune reports; the grids hold one block per
  * item. */

@@ -1209,9 +1209,13 @@ static pflb_status batch_build_items(pflb_batch *b) {
       cells += L->N;
     }
   }
-  // cells per bulk item: the launch shape's tile times its planes over 16
-  const int chunk =
-      (int)std::min(8192LL, std::max(64LL, (long long)b->dev.bx * b->dev.by * b->dev.lz / 16 / 64 * 64));
+  // Cells per bulk item: the launch shape's tile times its planes over 16, and a
+  // quarter of that at FP64, where a block is one warp and every further 32
+  // cells of an item add their whole time to the step.
+  const bool dp = b->storage == PFLB_STORAGE_FP64;
+  const int nt = dp ? 32 : 64;  // phase2_threads
+  const long long shape = (long long)b->dev.bx * b->dev.by * b->dev.lz / (dp ? 64 : 16);
+  const int chunk = (int)std::min(8192LL, std::max((long long)nt, shape / nt * nt));
   std::vector<int4> items;
   for (pflb::BatchGroup &g : b->groups) {
     auto add = [&](int l, int kind, int count, int per) {
@@ -1226,10 +1230,10 @@ static pflb_status batch_build_items(pflb_batch *b) {
     for (int l : g.lats) add(l, 0, (int)b->lats[l]->N, 1024);
     g.n1 = (int)items.size() - g.first1;
     g.first2 = (int)items.size();
-    for (int l : g.lats) add(l, 3, b->lats[l]->nw, 64);
+    for (int l : g.lats) add(l, 3, b->lats[l]->nw, nt);
     for (int l : g.lats) {
       const Lattice *L = b->lats[l];
-      if (L->bc_on) add(l, 4, 2 * L->ny * L->nz, 64);
+      if (L->bc_on) add(l, 4, 2 * L->ny * L->nz, nt);
     }
     for (int l : g.lats) add(l, 2, (int)b->lats[l]->N, chunk);
     g.n2 = (int)items.size() - g.first2;
