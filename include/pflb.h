@@ -81,9 +81,12 @@ enum { PFLB_FIELD_PHI = 0, PFLB_FIELD_RHO = 1, PFLB_FIELD_P = 2,
  *   PFLB_KERNEL_TWOPASS: a phi pass followed by a per-cell pass;
  *   PFLB_KERNEL_FUSED_TMA: the fused pass with h staged through shared
  *     memory by TMA (FP32 storage, nx a multiple of 4 and nx >= 64;
- *     otherwise PFLB_KERNEL_FUSED runs). */
+ *     otherwise PFLB_KERNEL_FUSED runs);
+ *   PFLB_KERNEL_MARCH: the z-marching kernel of the default kind at any size
+ *     and extent (FP32 storage, periodic x, nx a multiple of 4; otherwise the
+ *     two kernels run).  pflb_marches tells which of the two runs. */
 enum { PFLB_KERNEL_FUSED = 0, PFLB_KERNEL_TWOPASS = 1, PFLB_KERNEL_FUSED_TMA = 2,
-       PFLB_KERNEL_PIPE = 3 };
+       PFLB_KERNEL_PIPE = 3, PFLB_KERNEL_MARCH = 4 };
 
 /* Geometry, read during pflb_create only.
  *   solid       : host, nx*ny*nz bytes, nonzero = solid voxel.
@@ -251,6 +254,10 @@ pflb_status pflb_set_x_boundaries(pflb_lattice *L, const pflb_xbc *lo, const pfl
 
 /* The launch shape in effect: out = {kind, bx, by, lz}. */
 pflb_status pflb_get_kernel(const pflb_lattice *L, int out[4]);
+
+/* *marches = 1 if the lattice's next step runs the z-marching kernel of the
+ * kinds PFLB_KERNEL_PIPE and PFLB_KERNEL_MARCH, 0 if it runs another. */
+pflb_status pflb_marches(const pflb_lattice *L, int *marches);
 
 /* Autotuner of the planes per block (no counterpart in the paper: a launch
  * parameter of this library's kernels).  For the kernel kind in effect it

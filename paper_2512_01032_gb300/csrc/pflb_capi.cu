@@ -757,7 +757,7 @@ pflb_status pflb_set_kernel(pflb_lattice *L, int kind, int bx, int by, int lz) {
   pflb_status s = check_lattice(L);
   if (s != PFLB_OK) return s;
   if (kind != PFLB_KERNEL_FUSED && kind != PFLB_KERNEL_TWOPASS && kind != PFLB_KERNEL_FUSED_TMA &&
-      kind != PFLB_KERNEL_PIPE)
+      kind != PFLB_KERNEL_PIPE && kind != PFLB_KERNEL_MARCH)
     return fail(PFLB_ERR_ARG, "unknown kernel");
   if (lz < -1) return fail(PFLB_ERR_ARG, "lz must be > 0, 0 (keep) or -1 (automatic)");
   const int nbx = bx > 0 ? bx : L->bx, nby = by > 0 ? by : L->by;
@@ -878,13 +878,22 @@ pflb_status pflb_get_kernel(const pflb_lattice *L, int out[4]) {
   if (!out) return fail(PFLB_ERR_ARG, "null output");
   const bool tma = L->kernel == PFLB_KERNEL_FUSED_TMA && L->p.storage == PFLB_STORAGE_FP32 &&
                    L->tma_ok && !L->bc_on;
-  const bool pipe = L->kernel == PFLB_KERNEL_PIPE;
+  const bool pipe = L->kernel == PFLB_KERNEL_PIPE || L->kernel == PFLB_KERNEL_MARCH;
   // the kind that runs: the TMA kernel falls back to the fused one where it
-  // does not apply
+  // does not apply, the march to the two-phase step
   out[0] = pipe || tma || L->kernel == PFLB_KERNEL_TWOPASS ? L->kernel : PFLB_KERNEL_FUSED;
+  if (L->kernel == PFLB_KERNEL_MARCH && !pflb::pipe_kernel_runs(*L)) out[0] = PFLB_KERNEL_PIPE;
   out[1] = tma ? 32 : (pipe ? 32 : L->bx);
   out[2] = tma ? 8 : (pipe ? 4 : L->by);
   out[3] = L->lz;
+  return PFLB_OK;
+}
+
+pflb_status pflb_marches(const pflb_lattice *L, int *marches) {
+  pflb_status s = check_lattice(L);
+  if (s != PFLB_OK) return s;
+  if (!marches) return fail(PFLB_ERR_ARG, "null output");
+  *marches = pflb::pipe_kernel_runs(*L) ? 1 : 0;
   return PFLB_OK;
 }
 

@@ -107,14 +107,18 @@ struct BatchDev {
 
 // The pipelined step kernel runs with periodic x and nx a multiple of 4, so
 // that its 16-byte row chunks and 4-byte flag words are aligned.
-inline bool pipe_layout_ok(const Lattice &L) { return !L.bc_on && L.nx % 4 == 0; }
+inline bool pipe_layout_ok(const Lattice &L) {
+  return L.p.storage == PFLB_STORAGE_FP32 && !L.bc_on && L.nx % 4 == 0;
+}
 // The default kind runs the pipelined march where it pays and its layout allows
-// it, and the two-phase step elsewhere.
+// it, PFLB_KERNEL_MARCH wherever the layout does, and both the two-phase step
+// elsewhere.
 inline bool pipe_kernel_runs(const Lattice &L) {
-  return L.kernel == PFLB_KERNEL_PIPE && L.march && pipe_layout_ok(L);
+  return ((L.kernel == PFLB_KERNEL_PIPE && L.march) || L.kernel == PFLB_KERNEL_MARCH) &&
+         pipe_layout_ok(L);
 }
 inline bool phase_kernel_runs(const Lattice &L) {
-  return L.kernel == PFLB_KERNEL_PIPE && !pipe_kernel_runs(L);
+  return (L.kernel == PFLB_KERNEL_PIPE || L.kernel == PFLB_KERNEL_MARCH) && !pipe_kernel_runs(L);
 }
 
 // Accumulator of diagnostic step d (d = 2: the field pass), and the folded record.

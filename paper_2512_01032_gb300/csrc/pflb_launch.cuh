@@ -191,7 +191,9 @@ static cudaError_t launch_pipe_f(Lattice &L, Args<S, R> &a) {
   if (e != cudaSuccess) return e;
   const dim3 grid((L.nx + PP_BX - 1) / PP_BX, (L.ny + PP_BY - 1) / PP_BY,
                   (L.nz + L.lz - 1) / L.lz);
-  // the wall nodes of each block, listed for the planes per block in effect
+  // the wall nodes of each block, listed for the planes per block in effect (a
+  // list for another depth would have blocks update other blocks' nodes)
+  if (L.nw > 0 && (!L.wl || L.wl_lz != L.lz)) return cudaErrorInvalidValue;
   a.wl = L.nw > 0 ? L.wl : nullptr;
   a.wl_start = L.nw > 0 ? L.wl_start : nullptr;
   k_pipe<S, R, ODD, DIAG, FORCE><<<grid, PP_NT, sizeof(PipeSmem<S, R>), L.stream>>>(a);

@@ -21,7 +21,7 @@ OK, ERR_ARG, ERR_OOM, ERR_CUDA, ERR_NAN, ERR_TIMEOUT, ERR_BUDGET, ERR_STATE = ra
 STORAGE_FP64, STORAGE_FP32, STORAGE_FP16, STORAGE_BF16 = 0, 1, 2, 3
 FIELD_PHI, FIELD_RHO, FIELD_P, FIELD_UX, FIELD_UY, FIELD_UZ = range(6)
 FIELDS = {"phi": 0, "rho": 1, "P": 2, "ux": 3, "uy": 4, "uz": 5}
-KERNEL_FUSED, KERNEL_TWOPASS, KERNEL_FUSED_TMA, KERNEL_PIPE = 0, 1, 2, 3
+KERNEL_FUSED, KERNEL_TWOPASS, KERNEL_FUSED_TMA, KERNEL_PIPE, KERNEL_MARCH = 0, 1, 2, 3, 4
 
 STATUS_NAMES = {0: "OK", 1: "ERR_ARG", 2: "ERR_OOM", 3: "ERR_CUDA", 4: "ERR_NAN",
                 5: "ERR_TIMEOUT", 6: "ERR_BUDGET", 7: "ERR_STATE"}
@@ -173,6 +173,8 @@ def load(build_if_missing: bool = True):
     lib.pflb_selftest_wait_timeout.restype = st
     lib.pflb_get_kernel.argtypes = [C.c_void_p, _P(C.c_int)]
     lib.pflb_get_kernel.restype = st
+    lib.pflb_marches.argtypes = [C.c_void_p, _P(C.c_int)]
+    lib.pflb_marches.restype = st
     lib.pflb_tune.argtypes = [C.c_void_p, C.c_int, _P(C.c_int)]
     lib.pflb_tune.restype = st
     lib.pflb_step.argtypes = [C.c_void_p, C.c_int64]
@@ -414,6 +416,12 @@ class Lattice:
         lz = C.c_int(0)
         _check(self._lib.pflb_tune(self._h, int(trial_steps), C.byref(lz)))
         return lz.value
+
+    def marches(self) -> bool:
+        """Whether the next step runs the z-marching kernel."""
+        m = C.c_int()
+        _check(self._lib.pflb_marches(self._h, C.byref(m)))
+        return m.value != 0
 
     def step(self, n=1):
         _check(self._lib.pflb_step(self._h, int(n)))
