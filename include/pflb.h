@@ -260,7 +260,10 @@ pflb_status pflb_get_kernel(const pflb_lattice *L, int out[4]);
 pflb_status pflb_marches(const pflb_lattice *L, int *marches);
 
 /* Autotuner of the planes per block (no counterpart in the paper: a launch
- * parameter of this library's kernels).  For the kernel kind in effect it
+ * parameter of this library's marching kernels: PFLB_KERNEL_FUSED and
+ * PFLB_KERNEL_FUSED_TMA, and the default kind where pflb_marches says 1.  The
+ * two-phase and the two-pass step have no depth: there the steps are taken
+ * and the depth that is kept changes nothing).  For the kernel kind in effect it
  * times trial_steps steps at each of a fixed set of depths (the automatic
  * choice, 4, 6, 8, 10, 12, 16, 24, 32 planes, those not above nz) on the
  * lattice itself, keeps the fastest (as pflb_set_kernel with that lz) and
@@ -386,7 +389,8 @@ pflb_status pflb_fields_noalloc(int nx, int ny, int nz, const float *h_dev, cons
  * per block (a range of one lattice's cells, wall nodes or boundary cells), so
  * that small lattices that could not fill the GPU on their own share it and a
  * group's state stays in L2 from step to step.  Larger lattices are stepped
- * one after the other by their own kernels.  No work item reads another
+ * one after the other by the kernels of the default kind.  (The kind that
+ * pflb_set_kernel chose is for a lattice's own steps.)  No work item reads another
  * lattice, so a lattice's result does not depend on what it is batched with:
  * it is bit-identical to the same lattice in a batch of its own.  Against
  * pflb_step on that lattice it agrees to rounding (the kernels are compiled
@@ -407,6 +411,7 @@ pflb_status pflb_batch_create(pflb_lattice *const *lattices, int count, void *cu
 pflb_status pflb_batch_set_launch(pflb_batch *b, int bx, int by, int lz, int blocks_per_sm);
 
 /* Autotuner: times trial_steps steps of each of a fixed set of launch shapes
+ * (of no effect on lattices of 131072 cells and more)
  * on the batch itself (the steps are real steps of every lattice), keeps the
  * fastest and returns it in best (bx, by, lz, blocks per SM) if not NULL. */
 pflb_status pflb_batch_tune(pflb_batch *b, int trial_steps, int best[4]);

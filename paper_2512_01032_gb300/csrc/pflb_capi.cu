@@ -137,6 +137,7 @@ size_t h_slots_of(int storage) { return storage_bytes(storage) == 2 ? 20 : 19; }
 // 384 x 128 x 128 (478 MB, 3.1 % wall nodes) 426 / 426, 500 x 120 x 120 (547
 // MB) 509 / 494, sessile 176^3 380 / 374.  At 16-bit storage the two phases are
 // faster throughout (drop 192^3 368 / 362, channel 380 x 130 x 130 534 / 337).
+// Near the line the rule is up to 2 % wrong: the 176^3 sessile lattice marches.
 bool march_pays(const Lattice *L) {
   if (L->p.storage != PFLB_STORAGE_FP32) return false;
   int dev = 0, l2 = 0;
@@ -1381,15 +1382,21 @@ static pflb_status batch_run(pflb_batch *b, int64_t nsteps, bool diag_last) {
         }
       }
   }
+  // Larger lattices: their own kernels, on the batch stream and by the default
+  // kind, as the groups step theirs, so that a lattice's kind does not change
+  // what a batch computes.
   for (int l : b->alone) {
     Lattice *L = b->lats[l];
-    const cudaStream_t own = L->stream;
+    const cudaStream_t stream = L->stream;
+    const int kind = L->kernel;
     L->stream = b->dev.stream;
+    if (kind != PFLB_KERNEL_MARCH) L->kernel = PFLB_KERNEL_PIPE;
     L->in_batch = true;
-    cudaError_t e = cudaSuccess;
+    cudaError_t e = ensure_wall_lists(L, L->stream);
     for (int64_t t = 0; t < nsteps && e == cudaSuccess; ++t)
       e = do_step(L, diag_last && t == nsteps - 1);
-    L->stream = own;
+    L->stream = stream;
+    L->kernel = kind;
     L->in_batch = false;
     BCK(b, e);
   }

@@ -98,10 +98,12 @@ def single(name, storage, diag, tmp):
     return d
 
 
-def batch(storage, tmp):
+def batch(storage, tmp, kind=3):
     from paper_2512_01032_gb300 import pflb
     lats = [_lattice(n, storage) for n in BATCH]
     lats[0].step(1)  # the other A-A parity
+    for L in lats:
+        L.set_kernel(kind)
     B = pflb.Batch(lats)
     out = {}
     for steps, last in ((3, False), (4, True)):
@@ -130,4 +132,11 @@ def test_steps_keep_their_bits(name, storage, diag, tmp_path):
 @pytest.mark.parametrize("storage", STORAGES)
 def test_batch_steps_keep_their_bits(storage, tmp_path):
     got, want = batch(storage, tmp_path), _golden()
+    assert [k for k in got if got[k] != want[k]] == []
+
+
+@pytest.mark.parametrize("kind", [0, 1, 2, 4])
+def test_a_lattice_s_kind_does_not_change_a_batch(kind, tmp_path):
+    """Small lattices in groups and large ones by themselves alike."""
+    got, want = batch("fp32", tmp_path, kind), _golden()
     assert [k for k in got if got[k] != want[k]] == []
