@@ -49,7 +49,7 @@ CLOCK_WINDOW_S = 1.0  # untimed load before the timed region, for the clock reco
 KERNEL_SOURCES = ("pflb_kernels.cuh", "pflb_model.cuh", "pflb_launch.cuh", "pflb_phase.cuh",
                   "pflb_f32.cu")
 KERNEL_NAMES = {0: "k_fused", 1: "k_phi + k_cell", 2: "k_fused_async",
-                3: "k_phase1 + k_phase2"}
+                3: "k_phase1 + k_phase2", 4: "k_pipe"}
 KERNEL_TEXT = {0: "fused z-marching, direct loads", 1: "phi pass + per-cell pass",
                2: "fused z-marching, h staged by TMA",
                3: "two kernels, phi of every cell and then the update"}
@@ -62,30 +62,6 @@ def kernel_source_hash() -> str:
     for f in KERNEL_SOURCES:
         h.update(open(os.path.join(ROOT, "paper_2512_01032_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
-
-
-BATCH_SOURCES = ("pflb_phase.cuh", "pflb_kernels.cuh", "pflb_model.cuh", "pflb_launch.cuh",
-                 "pflb_bf16.cu")
-
-
-def batch_source_hash() -> str:
-    h = hashlib.sha256()
-    for f in BATCH_SOURCES:
-        h.update(open(os.path.join(ROOT, "paper_2512_01032_gb300", "csrc", f), "rb").read())
-    return h.hexdigest()[:16]
-
-
-def recorded_batch_traffic(storage, fluid):
-    """DRAM bytes per launch of the batch kernel, from the committed ncu
-    summary of a smaller case scaled by fluid cells, if it was taken on the
-    current sources at this storage."""
-    try:
-        d = json.load(open(os.path.join(ROOT, "profiles", "k_batch_channels8_bf16_traffic.json")))
-    except Exception:
-        return None
-    if d.get("batch_source_hash") != batch_source_hash() or d.get("storage") != storage:
-        return None
-    return d["dram_bytes_per_fluid_cell"] * fluid
 
 
 def hbm_peak():
@@ -384,8 +360,7 @@ def main_channels(args):
                        "l2": "inputs larger than L2 (no flush)"},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak,
-                         "traffic": recorded_batch_traffic(storage, fluid),
-                         "traffic_note": "ncu capture of 8 of the lattices, scaled by fluid cells",
+                         "traffic": None,
                          "peak_kind": f"{peak_kind} copy bandwidth (MEASURED_PEAKS hbm_gbs)",
                          "algorithmic_bytes_per_cell": ALGO_BYTES[storage],
                          "kernel": "k_batch_phase1 + k_batch_phase2"},

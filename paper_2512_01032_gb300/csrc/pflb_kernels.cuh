@@ -31,12 +31,6 @@ enum { MODE_STEP = 0, MODE_MACRO = 1 };
 // per direction with fixed roundings (collide's RN, FP32 arithmetic only).
 enum { COLL_FIXED = -1, COLL_PLAIN = 0, COLL_PAIRS = 1, COLL_X2 = 2, COLL_X2_NOF = 3 };
 
-// Blocks of 256 threads per SM the batch kernel is compiled for (sets its
-// register cap: 128).
-#ifndef PFLB_MIN_BLOCKS
-#define PFLB_MIN_BLOCKS 2
-#endif
-
 // Register cap of the plain fused kernel.  At 96 registers five 128-thread
 // blocks fit on an SM (20 warps instead of the 16 that 128 registers allow);
 // the FP32 and 16-bit instantiations then spill 36-52 bytes per thread, and

@@ -11,7 +11,7 @@
 // kernels the second read costs no DRAM traffic.  Measured (GB300, us per
 // step, against the march, or the fused kernel where that could not run):
 // FP32 drop 32^3 6.1 (10.3), sessile 64^3 14.6 (32.4), slit 1024 x 64 x 4 14.9
-// (31.7), constricted duct w = 48 29 (56), channel 251 x 67 x 67 75 (153), sessile
+// (31.7), constricted duct w = 48 29 (56), channel 251 x 67 x 67 87 (153), sessile
 // 128^3 136 (152); BF16 sessile 128^3 109 (138); FP64 sessile 64^3 303 (516).
 // What bounds it: at 128^3 FP32 phase 1 takes 28.7 us, the copy bandwidth, and
 // phase 2 runs at 82 to 90 % of it; at 16-bit storage the latency of the loads
@@ -37,10 +37,12 @@ template <class R>
 __host__ __device__ constexpr int phase2_threads() {
   return sizeof(R) == 8 ? 32 : 64;
 }
-// Phase-2 blocks per SM.  With 7 a thread has 144 registers, enough for all
-// loads of a cell (19 phi, 19 g, 19 h) to be in flight at once; more warps with
-// fewer registers are slower (BF16 sessile 128^3: 7 blocks 108.7 us per step, 8
-// blocks 112.6, 9 blocks 111.6; FP32 141.8, 141.8, 150.3).
+// Phase-2 blocks per SM that the compiler is asked for.  7 and 8 both give a
+// thread 128 registers (14 warps put four on a quarter of the SM), with which
+// nearly all loads of a cell (19 phi, 19 g, 19 h) are in flight at once; spill
+// stores are 0 to 8 bytes in even FP32 and BF16 steps, 68 to 92 in odd ones, 44
+// to 280 with diagnostics.  Sessile 128^3, us per step at 6 / 7 / 8 / 9 blocks:
+// FP32 154 / 142 / 142 / 150, BF16 134 / 109 / 113 / 112.
 template <class R>
 __host__ __device__ constexpr int phase2_blocks() {
   return sizeof(R) == 8 ? 8 : 7;
