@@ -166,8 +166,9 @@ int resolve_lz(Lattice *L) {
 // chunks alternating from both ends: chunk c < ceil(n/2) is block row 2c,
 // the others 2 (n - 1 - c) + 1).  Copied on stream st (the lattice's
 // stream once created, so that steps queued before use the previous lists);
-// copies from pageable memory have read the host vectors on return.
-cudaError_t ensure_wall_lists(Lattice *L, cudaStream_t st) {
+// copies from pageable memory have read the host vectors on return.  Host
+// memory that runs out is an error like the device's, not an exception.
+cudaError_t ensure_wall_lists(Lattice *L, cudaStream_t st) try {
   if (!L->wl || L->nw == 0 || L->wl_lz == L->lz || !pflb::pipe_kernel_runs(*L)) return cudaSuccess;
   const int lz = L->lz, gx = (L->nx + 31) / 32, gy = (L->ny + 3) / 4;
   const int nch = (L->nz + lz - 1) / lz;
@@ -192,6 +193,8 @@ cudaError_t ensure_wall_lists(Lattice *L, cudaStream_t st) {
                         cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) L->wl_lz = lz;
   return e;
+} catch (const std::bad_alloc &) {
+  return cudaErrorMemoryAllocation;
 }
 
 // Blocks of the pipelined grid at one plane per block (the size of wl_start).
