@@ -1,7 +1,6 @@
 """Steps in FP32 arithmetic keep their bits: checkpoints after a few steps
 against SHA-256 digests (golden/step_digests.json) taken on a GB300 from the
-kernels that stepped these lattices first, the marching kernels of earlier
-builds (commit ea09c90).
+marching kernels, which stepped these lattices first (commit ea09c90).
 
 The switch of the mobility correction (Eq. 4) turns one rounding into 1e-3 of
 phi at an interface cell within tens of steps, so a result that is the same to
